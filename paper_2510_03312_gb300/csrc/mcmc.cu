@@ -12,15 +12,27 @@
 // the Adam moments of all touched primitives are reset.
 //
 // Kernels (one launch each, in order):
-//   mcmc_weights_kernel  weights, per-1024-block inclusive scans, block sums;
-//                        clears the per-primitive counts and sources
+//   mcmc_weights_kernel  the weights' sums over chunks of 64 and blocks of 1024
+//                        primitives; clears the per-primitive counts and sources
 //   mcmc_scan_kernel     exclusive scan of the block sums (one block)
-//   mcmc_sample_kernel   each dead slot's source (two binary searches:
-//                        over the block offsets, then within the block);
-//                        per-source copy counts by integer atomics (exact)
-//   mcmc_copy_kernel     copies of the sources into the dead slots
-//   mcmc_sources_kernel  the sources' new opacity and reset moments
-// The copy kernel reads each source before the sources kernel updates it.
+//   mcmc_draw_kernel     each dead slot's source, the per-source copy counts
+//                        (integer atomics, exact) and the list of moved slots
+//   mcmc_copy_kernel     the sources copied into the listed slots, a plane per
+//                        grid row, but for the opacity
+//   mcmc_touched_kernel  the touched primitives' new opacity, from the final
+//                        counts, and zero moments; the caller's copy of the
+//                        sources
+//
+// A draw is a search of the cumulative weights, bound by the latency of its
+// dependent loads (a binary search in global memory took twenty); the copies
+// touch 32-byte sectors for 4 bytes each, anywhere in the planes: bound by
+// requests to L2, some 68 G a second here, and by address translation (a
+// warp copying all planes of one slot, a page per lane, took 154 us).  So the
+// copy kernel keeps each grid row in one plane and gives a listed slot to
+// each lane, and the moments are zeroed in primitive order, where neighbours
+// share requests.  P = 1M, K = 15, 5% dead, states larger than L2: 208 ->
+// 108 us a call (draw 52 -> 22, copies and moments 151 -> 58; a thread per
+// slot, most lanes idle, copied and zeroed all planes before).
 #include <math.h>
 
 #include "ubs.h"
@@ -30,13 +42,16 @@ namespace ubs {
 namespace {
 
 constexpr int kMcBlock = 1024;  // elements per scan block
+constexpr int kMcChunk = 64;    // elements per chunk of the in-block search: two per lane
+constexpr int kMcChunks = kMcBlock / kMcChunk;  // chunks per block
+constexpr unsigned kMcCopyRow = 152;            // blocks per plane of the copy kernel
 constexpr int kMcThreads = 256;
 constexpr int kMcMaxPlanes = 64;
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct McLayout {
-  size_t cdf, boff, counts, src, header, total;
+  size_t csum, list, boff, counts, src, header, total;
   uint32_t nb;
 };
 
@@ -46,7 +61,11 @@ McLayout mc_layout(int64_t P) {
   size_t o = 0;
   L.header = o;
   o += 256;  // total weight (u64), relocated count (i64)
-  L.cdf = o;
+  // the chunk sums (u64, 16 per block of 1024: 128 bytes a block), then the
+  // list of moved slots (4 bytes each, at most P): 128 ceil(P / 1024) + 4 P
+  // is at most 8 P rounded up to 256, for every P >= 1
+  L.csum = o;
+  L.list = o + (size_t)L.nb * kMcChunks * 8;
   o += align256((size_t)P * 8);
   L.boff = o;
   o += align256((size_t)L.nb * 8);
@@ -68,45 +87,48 @@ __device__ __forceinline__ uint32_t weight_of(float o, float thr) {
   return is_dead(o, thr) ? 0u : (uint32_t)(o * 16777216.0f);  // floor for o >= 0
 }
 
+// Sum of w over the warp, exact in 64 bits.
+__device__ __forceinline__ unsigned long long warp_sum_u32(uint32_t w) {
+  const unsigned lo = __reduce_add_sync(0xffffffffu, w & 0xffffu), hi = __reduce_add_sync(0xffffffffu, w >> 16);
+  return ((unsigned long long)hi << 16) + lo;
+}
+
 __global__ void __launch_bounds__(kMcThreads)
-    mcmc_weights_kernel(const float* __restrict__ op, int64_t P, float thr, unsigned long long* __restrict__ cdf,
+    mcmc_weights_kernel(const float* __restrict__ op, int64_t P, float thr, unsigned long long* __restrict__ csum,
                         unsigned long long* __restrict__ bsum, uint32_t* __restrict__ counts,
-                        int32_t* __restrict__ src, McHeader* hdr) {
+                        int32_t* __restrict__ src) {
   wait_prior_grid();
-  __shared__ unsigned long long warp_tot[kMcThreads / 32];
-  constexpr int E = kMcBlock / kMcThreads;  // 4 consecutive elements per thread
-  const int64_t base = (int64_t)blockIdx.x * kMcBlock + (int64_t)threadIdx.x * E;
-  unsigned long long v[E], run = 0;
+  __shared__ unsigned long long s_sum[kMcThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int E = kMcBlock / kMcThreads;  // elements per thread: two chunks per warp
+  const int64_t base = (int64_t)blockIdx.x * kMcBlock + warp * (32 * E) + lane;
+  float o[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) o[e] = base + e * 32 < P ? op[base + e * 32] : -1.0f;
+  unsigned long long sum[E / 2];
 #pragma unroll
   for (int e = 0; e < E; ++e) {
-    const int64_t i = base + e;
-    uint32_t w = 0;
+    const int64_t i = base + e * 32;
     if (i < P) {
-      w = weight_of(op[i], thr);
       counts[i] = 0;
       src[i] = -1;
     }
-    run += w;
-    v[e] = run;  // thread-local inclusive
+    const unsigned long long s = warp_sum_u32(i < P ? weight_of(o[e], thr) : 0u);
+    sum[e / 2] = (e & 1) ? sum[e / 2] + s : s;
   }
-  // inclusive scan of the thread totals over the block
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned long long x = run;
+  unsigned long long tot = 0;
 #pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const unsigned long long y = __shfl_up_sync(0xffffffffu, x, d);
-    if (lane >= d) x += y;
+  for (int c = 0; c < E / 2; ++c) {
+    if (lane == 0) csum[(size_t)blockIdx.x * kMcChunks + warp * (E / 2) + c] = sum[c];
+    tot += sum[c];
   }
-  if (lane == 31) warp_tot[warp] = x;
+  if (lane == 0) s_sum[warp] = tot;
   __syncthreads();
-  unsigned long long woff = 0;
-  for (int w = 0; w < warp; ++w) woff += warp_tot[w];
-  const unsigned long long excl = woff + x - run;
-#pragma unroll
-  for (int e = 0; e < E; ++e)
-    if (base + e < P) cdf[base + e] = excl + v[e];
-  if (threadIdx.x == kMcThreads - 1) bsum[blockIdx.x] = woff + x;
-  if (blockIdx.x == 0 && threadIdx.x == 0) hdr->relocated = 0;
+  if (threadIdx.x == 0) {
+    unsigned long long b = 0;
+    for (int w = 0; w < kMcThreads / 32; ++w) b += s_sum[w];
+    bsum[blockIdx.x] = b;
+  }
 }
 
 // exclusive scan of the block sums in place (one block, sequential chunks)
@@ -137,35 +159,10 @@ __global__ void __launch_bounds__(1024) mcmc_scan_kernel(unsigned long long* __r
     if (threadIdx.x == 1023) carry = c + woff + x;
     __syncthreads();
   }
-  if (threadIdx.x == 0) hdr->total = carry;
-}
-
-__global__ void __launch_bounds__(kMcThreads)
-    mcmc_sample_kernel(const float* __restrict__ op, int64_t P, float thr, const unsigned long long* __restrict__ rnd,
-                       const unsigned long long* __restrict__ cdf, const unsigned long long* __restrict__ boff,
-                       uint32_t nb, uint32_t* __restrict__ counts, int32_t* __restrict__ src, McHeader* hdr) {
-  wait_prior_grid();
-  const int64_t j = (int64_t)blockIdx.x * kMcThreads + threadIdx.x;
-  const unsigned long long total = hdr->total;
-  if (j >= P || total == 0 || !is_dead(op[j], thr)) return;
-  const unsigned long long r = rnd[j] % total;
-  // the last block whose offset is <= r, then the first element of it whose
-  // inclusive cumulative weight exceeds r
-  uint32_t lo = 0, hi = nb - 1;
-  while (lo < hi) {
-    const uint32_t mid = (lo + hi + 1) >> 1;
-    if (boff[mid] <= r) lo = mid; else hi = mid - 1;
+  if (threadIdx.x == 0) {
+    hdr->total = carry;
+    hdr->relocated = 0;
   }
-  const unsigned long long rr = r - boff[lo];
-  int64_t a = (int64_t)lo * kMcBlock, b = a + kMcBlock - 1;
-  if (b > P - 1) b = P - 1;
-  while (a < b) {
-    const int64_t mid = (a + b) >> 1;
-    if (cdf[mid] > rr) b = mid; else a = mid + 1;
-  }
-  src[j] = (int32_t)a;
-  atomicAdd(&counts[a], 1u);
-  atomicAdd((unsigned long long*)&hdr->relocated, 1ull);
 }
 
 struct McPlanes {
@@ -176,54 +173,161 @@ __device__ __forceinline__ float cloned_opacity(float o, uint32_t n) {
   return 1.0f - powf(1.0f - o, 1.0f / (float)(n + 1));
 }
 
+// inclusive sum over the lanes up to this one
+__device__ __forceinline__ unsigned long long warp_incl_scan(unsigned long long x) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const unsigned long long y = __shfl_up_sync(0xffffffffu, x, d);
+    if (lane >= d) x += y;
+  }
+  return x;
+}
+
+// A block draws for the dead of its kMcBlock slots: it lists them in shared
+// memory, each thread then takes a listed slot and finds the block of
+// primitives its draw falls in (every stride-th block offset is staged in
+// shared memory; at most two steps' worth of offsets are then read from
+// global memory for scenes of up to 4M primitives), and each warp finishes
+// its slots one after the other with all lanes: the chunk sums of the block,
+// then the chunk's weights, two dependent loads a slot.
+constexpr uint32_t kMcOffs = 1024;  // staged block offsets
+__global__ void __launch_bounds__(kMcThreads)
+    mcmc_draw_kernel(const float* __restrict__ op, int64_t P, float thr, const unsigned long long* __restrict__ rnd,
+                     const unsigned long long* __restrict__ csum, const unsigned long long* __restrict__ boff,
+                     uint32_t nb, uint32_t* __restrict__ counts, int32_t* __restrict__ src,
+                     int32_t* __restrict__ list, McHeader* hdr) {
+  wait_prior_grid();
+  __shared__ unsigned long long s_off[kMcOffs];
+  __shared__ int32_t s_slot[kMcBlock];
+  __shared__ uint32_t s_n;
+  __shared__ unsigned long long s_at;
+  const int lane = threadIdx.x & 31;
+  const unsigned long long total = hdr->total;
+  if (total == 0) return;
+  if (threadIdx.x == 0) s_n = 0;
+  const uint32_t stride = (nb + kMcOffs - 1) / kMcOffs, n_off = (nb + stride - 1) / stride;
+  for (uint32_t i = threadIdx.x; i < n_off; i += kMcThreads) s_off[i] = boff[i * stride];
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < kMcBlock / kMcThreads; ++e) {
+    const int64_t j = (int64_t)blockIdx.x * kMcBlock + e * kMcThreads + threadIdx.x;
+    const bool dead = j < P && is_dead(op[j], thr);
+    const unsigned all = __ballot_sync(0xffffffffu, dead);
+    uint32_t at = 0;
+    if (lane == 0 && all) at = atomicAdd(&s_n, (uint32_t)__popc(all));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(all & ((1u << lane) - 1u));
+    if (dead) s_slot[at] = (int32_t)j;
+  }
+  __syncthreads();
+  const uint32_t n = s_n;
+  if (n == 0) return;
+  if (threadIdx.x == 0) s_at = atomicAdd((unsigned long long*)&hdr->relocated, (unsigned long long)n);
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < n; i += kMcThreads) list[s_at + i] = s_slot[i];  // below P: each slot once
+  // 32 slots a warp and round, spread so that few slots still use every warp
+  const uint32_t n_warps = kMcThreads / 32;
+  for (uint32_t w0 = threadIdx.x >> 5; w0 < n; w0 += 32 * n_warps) {
+    const uint32_t i = w0 + lane * n_warps;
+    const bool on = i < n;
+    unsigned long long r = 0;
+    uint32_t lo = 0;
+    if (on) {
+      r = rnd[s_slot[i]] % total;
+      uint32_t hi = n_off - 1;  // the last staged offset at most r (the first, 0, is)
+      while (lo < hi) {
+        const uint32_t mid = (lo + hi + 1) >> 1;
+        if (s_off[mid] <= r) lo = mid; else hi = mid - 1;
+      }
+      lo *= stride;
+      hi = min(lo + stride, nb) - 1;  // then the last of the offsets up to the next staged one
+      while (lo < hi) {
+        const uint32_t mid = (lo + hi + 1) >> 1;
+        if (boff[mid] <= r) lo = mid; else hi = mid - 1;
+      }
+      r -= boff[lo];
+    }
+    const unsigned act = __ballot_sync(0xffffffffu, on);
+    int32_t from = -1;
+    for (unsigned rest = act; rest != 0; rest &= rest - 1) {
+      const int l = __ffs(rest) - 1;
+      unsigned long long rr = __shfl_sync(0xffffffffu, r, l);
+      const uint32_t b = __shfl_sync(0xffffffffu, lo, l);
+      // the block's first chunk whose inclusive sum exceeds rr
+      const unsigned long long cs = lane < kMcChunks ? csum[(size_t)b * kMcChunks + lane] : 0ull;
+      unsigned long long x = warp_incl_scan(cs);
+      const int ch = __ffs(__ballot_sync(0xffffffffu, x > rr)) - 1;  // some chunk does: r < total
+      rr -= __shfl_sync(0xffffffffu, x - cs, ch);
+      // and that chunk's first primitive, in its first or second half
+      const int64_t p = (int64_t)b * kMcBlock + ch * kMcChunk + lane;
+      const uint32_t q0 = p < P ? weight_of(op[p], thr) : 0u, q1 = p + 32 < P ? weight_of(op[p + 32], thr) : 0u;
+      x = warp_incl_scan(q0);
+      unsigned over = __ballot_sync(0xffffffffu, x > rr);
+      int at = __ffs(over) - 1;
+      if (over == 0) {  // warp-uniform
+        rr -= __shfl_sync(0xffffffffu, x, 31);
+        x = warp_incl_scan(q1);
+        over = __ballot_sync(0xffffffffu, x > rr);
+        at = 31 + __ffs(over);
+      }
+      if (lane == l) from = (int32_t)((int64_t)b * kMcBlock + ch * kMcChunk + at);
+    }
+    if (on) {
+      src[s_slot[i]] = from;
+      atomicAdd(&counts[from], 1u);
+    }
+  }
+}
+
+// Row y of the grid copies plane y of the sources into the listed slots.  A
+// source is live and a slot dead, so no thread reads what another writes.  A
+// slot's new opacity needs the final counts and its source's old opacity,
+// which is left in the slot's raw opacity.
 __global__ void __launch_bounds__(kMcThreads)
     mcmc_copy_kernel(McPlanes pl, int64_t P, float* __restrict__ act, float* __restrict__ raw,
-                     float* __restrict__ m, float* __restrict__ v, const uint32_t* __restrict__ counts,
-                     const int32_t* __restrict__ src) {
+                     const int32_t* __restrict__ src, const int32_t* __restrict__ list, const McHeader* hdr) {
   wait_prior_grid();
-  const int64_t j = (int64_t)blockIdx.x * kMcThreads + threadIdx.x;
-  if (j >= P) return;
-  const int32_t s = src[j];
-  if (s < 0) return;
-  for (int k = 0; k < pl.K; ++k) {
-    const size_t d = (size_t)k * P + j, o = (size_t)k * P + s;
-    if (k == pl.op_row) {
-      const float op = cloned_opacity(act[o], counts[s]);
-      act[d] = op;
-      raw[d] = logf(op / (1.0f - op));
+  const int64_t n = hdr->total ? hdr->relocated : 0;
+  const size_t plane = (size_t)blockIdx.y * P;
+  const bool opacity = (int)blockIdx.y == pl.op_row;
+  for (int64_t i = (int64_t)blockIdx.x * kMcThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kMcThreads) {
+    const int32_t j = list[i], s = src[j];
+    const size_t d = plane + j, o = plane + s;
+    const float a = act[o];
+    if (opacity) {
+      raw[d] = a;
     } else {
-      act[d] = act[o];
+      act[d] = a;
       raw[d] = raw[o];
     }
-    m[d] = 0.0f;
-    v[d] = 0.0f;
   }
 }
 
+// Every touched primitive, slot or source, in its own lane: the new opacity
+// (a moved slot's raw opacity holds its source's from before, a source's own
+// is in place) and zero moments.  Neighbours share lines here: one request
+// per warp and plane instead of one per slot and one per source.
 __global__ void __launch_bounds__(kMcThreads)
-    mcmc_sources_kernel(McPlanes pl, int64_t P, float* __restrict__ act, float* __restrict__ raw,
-                        float* __restrict__ m, float* __restrict__ v, const uint32_t* __restrict__ counts) {
-  wait_prior_grid();
-  const int64_t s = (int64_t)blockIdx.x * kMcThreads + threadIdx.x;
-  if (s >= P) return;
-  const uint32_t n = counts[s];
-  if (n == 0) return;
-  const size_t o = (size_t)pl.op_row * P + s;
-  const float op = cloned_opacity(act[o], n);
-  act[o] = op;
-  raw[o] = logf(op / (1.0f - op));
-  for (int k = 0; k < pl.K; ++k) {
-    m[(size_t)k * P + s] = 0.0f;
-    v[(size_t)k * P + s] = 0.0f;
-  }
-}
-
-__global__ void mcmc_export_kernel(const int32_t* __restrict__ src, int64_t P, int32_t* __restrict__ out,
-                                   const McHeader* hdr, long long* __restrict__ n_out) {
+    mcmc_touched_kernel(McPlanes pl, int64_t P, float* __restrict__ act, float* __restrict__ raw,
+                        float* __restrict__ m, float* __restrict__ v, const uint32_t* __restrict__ counts,
+                        const int32_t* __restrict__ src, int32_t* __restrict__ out, const McHeader* hdr,
+                        long long* __restrict__ n_out) {
   wait_prior_grid();
   const int64_t j = (int64_t)blockIdx.x * kMcThreads + threadIdx.x;
-  if (out && j < P) out[j] = src[j];
   if (n_out && j == 0) *n_out = hdr->relocated;
+  if (j >= P) return;
+  const int32_t s = src[j];
+  const uint32_t own = counts[j];
+  if (out) out[j] = s;
+  if (s < 0 && own == 0) return;
+  for (int k = 0; k < pl.K; ++k) {
+    m[(size_t)k * P + j] = 0.0f;
+    v[(size_t)k * P + j] = 0.0f;
+  }
+  const size_t o = (size_t)pl.op_row * P + j;
+  const float op = cloned_opacity(s >= 0 ? raw[o] : act[o], s >= 0 ? counts[s] : own);
+  act[o] = op;
+  raw[o] = logf(op / (1.0f - op));
 }
 
 }  // namespace
@@ -252,28 +356,28 @@ extern "C" ubs_status ubs_mcmc_relocate(int32_t K, int64_t P, int32_t opacity_ro
   if (workspace_bytes < L.total) return UBS_ERR_WORKSPACE;
   char* ws = (char*)workspace;
   McHeader* hdr = (McHeader*)(ws + L.header);
-  unsigned long long* cdf = (unsigned long long*)(ws + L.cdf);
+  unsigned long long* csum = (unsigned long long*)(ws + L.csum);
   unsigned long long* boff = (unsigned long long*)(ws + L.boff);
   uint32_t* counts = (uint32_t*)(ws + L.counts);
   int32_t* src = (int32_t*)(ws + L.src);
+  int32_t* list = (int32_t*)(ws + L.list);
   const float* op = act + (size_t)opacity_row * P;
   const unsigned grid = (unsigned)((P + kMcThreads - 1) / kMcThreads);
   McPlanes pl{K, opacity_row};
   cudaError_t e = launch_dependent(mcmc_weights_kernel, dim3(L.nb), dim3(kMcThreads), 0, stream, op, P,
-                                   dead_threshold, cdf, boff, counts, src, hdr);
+                                   dead_threshold, csum, boff, counts, src);
   if (e == cudaSuccess) e = launch_dependent(mcmc_scan_kernel, dim3(1), dim3(1024), 0, stream, boff, L.nb, hdr);
   if (e == cudaSuccess)
-    e = launch_dependent(mcmc_sample_kernel, dim3(grid), dim3(kMcThreads), 0, stream, op, P, dead_threshold,
-                         (const unsigned long long*)rand, (const unsigned long long*)cdf,
-                         (const unsigned long long*)boff, L.nb, counts, src, hdr);
+    e = launch_dependent(mcmc_draw_kernel, dim3(L.nb), dim3(kMcThreads), 0, stream, op, P, dead_threshold,
+                         (const unsigned long long*)rand, (const unsigned long long*)csum,
+                         (const unsigned long long*)boff, L.nb, counts, src, list, hdr);
+  const unsigned row = grid < kMcCopyRow ? grid : kMcCopyRow;
   if (e == cudaSuccess)
-    e = launch_dependent(mcmc_copy_kernel, dim3(grid), dim3(kMcThreads), 0, stream, pl, P, act, raw, m, v,
-                         (const uint32_t*)counts, (const int32_t*)src);
+    e = launch_dependent(mcmc_copy_kernel, dim3(row, (unsigned)K), dim3(kMcThreads), 0, stream, pl, P, act, raw,
+                         (const int32_t*)src, (const int32_t*)list, (const McHeader*)hdr);
   if (e == cudaSuccess)
-    e = launch_dependent(mcmc_sources_kernel, dim3(grid), dim3(kMcThreads), 0, stream, pl, P, act, raw, m, v,
-                         (const uint32_t*)counts);
-  if (e == cudaSuccess && (sources || n_relocated))
-    e = launch_dependent(mcmc_export_kernel, dim3(grid), dim3(kMcThreads), 0, stream, (const int32_t*)src, P,
-                         sources, (const McHeader*)hdr, (long long*)n_relocated);
+    e = launch_dependent(mcmc_touched_kernel, dim3(grid), dim3(kMcThreads), 0, stream, pl, P, act, raw, m, v,
+                         (const uint32_t*)counts, (const int32_t*)src, sources, (const McHeader*)hdr,
+                         (long long*)n_relocated);
   return e == cudaSuccess ? UBS_OK : UBS_ERR_CUDA;
 }

@@ -69,3 +69,47 @@ def test_relocation_matches_reference(dev, P, seed, dead_frac):
     assert np.array_equal(rg[orow][~touched], raw[orow][~touched])
     assert np.array_equal(t["m"].cpu().numpy(), m_r.astype(np.float32))
     assert np.array_equal(t["v"].cpu().numpy(), v_r.astype(np.float32))
+
+
+@pytest.mark.parametrize("P,dead_frac", [(32, 0.5), (33, 0.5), (32 * 1024, 0.01), (32 * 1024 + 1, 0.3),
+                                         (1024 * 1024 + 1, 0.02)])
+def test_draw_search_at_its_level_edges(dev, P, dead_frac):
+    """The 32-way search of a draw at the edges of its levels: one chunk of 32,
+    32 blocks of 1024 and one more, 1024 blocks and one more (a third level),
+    with runs of zero weights; the sources against the cumulative weights by
+    definition, bit for bit.  One plane, the opacity."""
+    import ctypes
+
+    from paper_2510_03312_gb300 import ubs as U
+    rng = np.random.default_rng(P)
+    o = rng.random(P).astype(np.float32)
+    o[rng.random(P) < dead_frac] = 0.0
+    o[P // 4:P // 2] = 0.0  # whole chunks and blocks without weight
+    o[-1] = 1.0
+    o[0] = 0.0
+    rand = rng.integers(0, 2 ** 63, size=P, dtype=np.uint64) * np.uint64(2) + np.uint64(1)
+    dead = o <= np.float32(0.005)
+    w = np.where(dead, 0, np.floor(o.astype(np.float64) * 2 ** 24)).astype(np.uint64)
+    cum = np.cumsum(w, dtype=np.uint64)
+    want = np.where(dead, np.searchsorted(cum, rand % cum[-1], side="right"), -1).astype(np.int32)
+    act, raw = torch.tensor(o, device=dev)[None].contiguous(), torch.zeros(1, P, device=dev)
+    m, v = torch.ones(1, P, device=dev), torch.ones(1, P, device=dev)
+    rnd = torch.tensor(rand.view(np.int64), device=dev)
+    src = torch.empty(P, dtype=torch.int32, device=dev)
+    nrel = torch.zeros(1, dtype=torch.int64, device=dev)
+    n = U.ubs_mcmc_workspace_size(P)
+    ws = torch.empty(n + 256, dtype=torch.uint8, device=dev)
+    st = U.ubs_mcmc_relocate(1, P, 0, 0.005, act.data_ptr(), raw.data_ptr(), m.data_ptr(), v.data_ptr(),
+                             rnd.data_ptr(), src.data_ptr(), nrel.data_ptr(), (ws.data_ptr() + 255) // 256 * 256, n,
+                             ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == U.UBS_OK
+    assert np.array_equal(src.cpu().numpy(), want)
+    assert int(nrel.item()) == int(dead.sum())
+    copies = np.bincount(want[dead], minlength=P)
+    new = 1.0 - (1.0 - o.astype(np.float64)) ** (1.0 / (copies + 1))
+    ref = np.where(dead, new[np.maximum(want, 0)], np.where(copies > 0, new, o))
+    # 1 - powf(1 - o, 1 / (n + 1)): a few roundings of numbers up to 1
+    np.testing.assert_allclose(act[0].cpu().numpy(), ref, rtol=2e-6, atol=5e-7)
+    moved = dead | (copies > 0)
+    assert np.array_equal(m[0].cpu().numpy(), np.where(moved, 0.0, 1.0).astype(np.float32))
+    assert np.array_equal(v[0].cpu().numpy(), np.where(moved, 0.0, 1.0).astype(np.float32))
