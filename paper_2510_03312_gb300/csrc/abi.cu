@@ -128,17 +128,35 @@ ubs_status make_layout(const ubs_problem* pr, Layout& L) {
   L.last = take((size_t)L.NPIX * 4);
   L.pairs = take((size_t)L.NPIX * 8);  // pairs with r < 1, then visited entries
   if (c.flags & kFlagSplit) {
-    // a split tile holds more than kSegLen instances, and its segments number
-    // at most its instances / kSegLen + 1: bounds from the capacity
-    L.seg_max_split = L.cap / kSegLen + 1;
-    L.seg_max_extra = L.cap / kSegLen + 1;
-    L.seg_slots = 2 * (L.cap / kSegLen) + 2;
+    // A split tile holds more than kSplitMin instances: their number, and
+    // that of their segments (n / length + 1 at most for a list of n), is
+    // bounded from the capacity.  The segments use the bytes set aside here
+    // and the counting variant's pair counts (which never splits); as many
+    // slots as these hold let the segments of the lists there are be short.
+    const size_t tile_px = (size_t)c.tile_w * (size_t)c.tile_h, at = L.pairs;
+    L.seg_max_split = L.cap / kSplitMin + 1;
+    const size_t aside = align256((size_t)L.seg_max_split * 16) + align256((size_t)L.NT * 4) +
+                         align256(2 * (size_t)L.seg_max_split * tile_px * 32) +
+                         align256(2 * (size_t)L.seg_max_split * 4) + 2 * align256((size_t)L.seg_max_split * 4);
+    const size_t end = o + aside;
+    o = at;
     L.split_list = take((size_t)L.seg_max_split * 16);
     L.tile_slot = take((size_t)L.NT * 4);
-    L.seg_buf = take((size_t)L.seg_slots * (size_t)c.tile_w * (size_t)c.tile_h * 32);
+    L.seg_end = take((size_t)L.seg_max_split * tile_px * 4);
+    L.split_term = take((size_t)L.seg_max_split * 4);
+    // 20 bytes of state per slot and pixel, an owner per slot and per extra
+    // segment; at least 2 seg_max_split - 1 slots fit in any case: 24 bytes a
+    // pixel with seg_end, of 32
+    const size_t slots = (end - o - 4 * 256) / (tile_px * 20 + 8);
+    const uint64_t most = (uint64_t)L.cap / kSegMin + L.seg_max_split;
+    L.seg_slots = L.seg_max_extra = (uint32_t)(slots < most ? slots : most);
+    L.seg_c = take((size_t)L.seg_slots * tile_px * 16);
+    L.seg_l = take((size_t)L.seg_slots * tile_px * 4);
     L.slot_owner = take((size_t)L.seg_slots * 4);
     L.ext_owner = take((size_t)L.seg_max_extra * 4);
-    L.split_term = take((size_t)L.seg_max_split * 4);
+    L.seg_safe = kSegMin;
+    while (L.seg_safe < kSplitMin && (uint64_t)L.cap / L.seg_safe + L.seg_max_split > L.seg_slots) L.seg_safe *= 2;
+    o = end;
   }
   L.total = o;
   return UBS_OK;

@@ -106,20 +106,28 @@ struct Layout {
   size_t Tfin, last, pairs;
   // long tile lists split across CTAs (UBS_FLAG_SPLIT_LISTS): the split
   // tiles [seg_max_split] x (tile, first slot, segments, first extra
-  // segment), each tile's first slot or ~0 [NT], and per (slot, pixel of
-  // the tile) 8 floats of segment state [seg_slots][tile pixels][8]
-  size_t split_list, tile_slot, seg_buf;
+  // segment), each tile's split index or ~0 [NT], per (slot, pixel of the
+  // tile) the segment's state: colour and T [seg_slots][tile pixels] x
+  // float4, last contributor and a flag [seg_slots][tile pixels] x u32, and
+  // per (split tile, pixel) the segment its walk ends in
+  size_t split_list, tile_slot, seg_c, seg_l, seg_end;
   size_t slot_owner;  // split tile of each slot [seg_slots]
   size_t ext_owner;   // split tile of each extra segment [seg_max_extra]
   size_t split_term;  // per split tile: the first segment after which every pixel had ended [seg_max_split]
   uint32_t seg_max_split, seg_max_extra, seg_slots;
+  uint32_t seg_safe;  // entries per segment for which the slots suffice whatever the lists
   size_t total;
 };
 
-// Tiles whose lists are longer than kSegLen entries are split into segments
-// of kSegLen entries (a multiple of every blend batch size) when
-// UBS_FLAG_SPLIT_LISTS is set.
-constexpr uint32_t kSegLen = 2048;
+// Tiles whose lists are longer than kSplitMin entries are split when
+// UBS_FLAG_SPLIT_LISTS is set, into segments of kSegMin (or the blend's batch,
+// where that is longer), 2, 4, .. times that, up to kSplitMin entries: the
+// shortest of which the workspace holds the state, which split_plan_kernel
+// finds from the number of long lists' sort chunks (Header::n_long) and
+// leaves in ctr[kCtrSegLen].
+constexpr uint32_t kSplitMin = 2048;
+constexpr uint32_t kSegMin = 128;
+constexpr uint32_t kSegEnded = 0x80000000u;  // flag beside the last contributor (a position below 2^31)
 constexpr uint32_t kFlagSplit = 16;
 constexpr uint32_t kFlagNoThresholds = 32;
 constexpr uint32_t kFlagChecked = 64;
@@ -143,6 +151,7 @@ constexpr int kGradFloats = 12;
 constexpr uint32_t kScanTiles = 1024;
 constexpr uint32_t kTileSub = 8;
 constexpr uint32_t kSortChunk = 512;
+constexpr int kCtrSegLen = 7;      // entries per segment of the split lists
 constexpr int kCtrSortItems = 8;   // header counter of the per-tile sort's next item
 constexpr int kCtrMergeItems = 9;  // and of the merge's
 constexpr uint32_t kVisBlocks = 1024;  // bound on the blocks of the binning's count walk

@@ -271,22 +271,26 @@ struct FwdArgs {
   const uint32_t* slot_owner;  // split index of each slot
   const uint32_t* ext_owner;   // split index of each extra segment
   uint32_t* split_term;        // per split tile: first segment after which every pixel had ended
-  float4* seg_buf;
-  uint32_t max_extra;
+  float4* seg_c;               // per (slot, pixel of the tile): colour and T
+  uint32_t* seg_l;             // and last contributor, with kSegEnded
+  uint32_t* seg_end;           // per (split tile, pixel): the segment its walk ends in
+  uint32_t max_extra, max_slots;  // grid bounds: CTAs of extra segments and of slots, each looping
 };
 
 // One tile g, by the whole CTA (every thread calls it).  With SPLIT it
 // walks only the list positions [wbeg, wend) of the tile and, when `slot`
 // is given, writes each pixel's state there (colour, T, last contributor
 // and whether the pixel terminated) instead of the image: the part of one
-// segment of a split list.
+// segment `seg` of a split list.  With `resume` (per pixel, the segment its
+// walk ends in) only the pixels ending in this segment are walked.
 // A segment k > 0 that learns (through `term`) that an earlier segment ended
 // every pixel of the tile stops: no pixel's result can use it.  A segment
 // whose walk ends every pixel records its index there.
 template <int TW, int TH, bool COUNT, bool SPLIT = false>
 __device__ __forceinline__ void fwd_tile(const FwdArgs& A, uint32_t g, FwdSmem<TW, TH>& sm, uint32_t wbeg = 0,
                                          uint32_t wend = 0xffffffffu, float4* slot = nullptr,
-                                         bool resume = false, uint32_t* term = nullptr, uint32_t seg = 0) {
+                                         uint32_t* slot_l = nullptr, const uint32_t* resume = nullptr,
+                                         uint32_t* term = nullptr, uint32_t seg = 0) {
   constexpr int NT = FwdSmem<TW, TH>::NT, BS = FwdSmem<TW, TH>::BS;
   const CfgDev& cfg = A.cfg;
   uint32_t start = A.tstart[g], end = A.tstart[g + 1];  // loaded while warp 0 finds the view
@@ -319,13 +323,12 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& A, uint32_t g, FwdSmem<T
   bool need0 = true, need1 = true;
   if constexpr (SPLIT) {
     if (resume) {  // a pixel whose walk ends in this segment resumes from its T and last contributor
-      const float4 a0 = slot[2 * (ly * TW + lx)], a1 = slot[2 * (ly * TW + lx) + 1];
-      const float4 b0 = slot[2 * ((ly + 4) * TW + lx)], b1 = slot[2 * ((ly + 4) * TW + lx) + 1];
-      need0 = __float_as_uint(a1.y) != 0u;
-      need1 = __float_as_uint(b1.y) != 0u;
-      T = make_float2(a0.w, b0.w);
-      last0 = __float_as_uint(a1.x);
-      last1 = __float_as_uint(b1.x);
+      const uint32_t l0 = slot_l[ly * TW + lx], l1 = slot_l[(ly + 4) * TW + lx];
+      need0 = resume[ly * TW + lx] == (seg | kSegEnded);
+      need1 = resume[(ly + 4) * TW + lx] == (seg | kSegEnded);
+      T = make_float2(need0 ? slot[ly * TW + lx].w : 1.0f, need1 ? slot[(ly + 4) * TW + lx].w : 1.0f);
+      last0 = l0;
+      last1 = l1;
       done0 = done0 || !need0;
       done1 = done1 || !need1;
     }
@@ -412,15 +415,14 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& A, uint32_t g, FwdSmem<T
   if constexpr (SPLIT) {
     if (term && __syncthreads_count(done0 && done1) == NT && threadIdx.x == 0) atomicMin(term, seg);
     if (slot) {  // one segment's state of the lane's two pixels (only the resumed ones when resuming)
-      float4* s0 = slot + 2 * (ly * TW + lx);
-      float4* s1 = slot + 2 * ((ly + 4) * TW + lx);
+      const int p0 = ly * TW + lx, p1 = (ly + 4) * TW + lx;
       if (need0) {
-        s0[0] = make_float4(C0.x, C1.x, C2.x, T.x);
-        s0[1] = make_float4(__uint_as_float(last0), __uint_as_float(done0 ? 1u : 0u), 0.0f, 0.0f);
+        slot[p0] = make_float4(C0.x, C1.x, C2.x, T.x);
+        slot_l[p0] = resume || !done0 ? last0 : last0 | kSegEnded;
       }
       if (need1) {
-        s1[0] = make_float4(C0.y, C1.y, C2.y, T.y);
-        s1[1] = make_float4(__uint_as_float(last1), __uint_as_float(done1 ? 1u : 0u), 0.0f, 0.0f);
+        slot[p1] = make_float4(C0.y, C1.y, C2.y, T.y);
+        slot_l[p1] = resume || !done1 ? last1 : last1 | kSegEnded;
       }
       return;
     }
@@ -455,9 +457,9 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& A, uint32_t g, FwdSmem<T
 
 // The grid form: one CTA per tile, in bin_sort's tile order where the lists
 // are dense.  With SPLIT a split tile's own CTA walks its first segment, and
-// A.max_extra more CTAs after the tiles' walk the later segments (those that
-// split_plan_kernel did not assign exit): started after the tiles, they can
-// find their tile already ended by its first segment, as dense tiles are.
+// A.max_extra more CTAs after the tiles' walk the later segments, each every
+// max_extra-th: started after the tiles, they can find their tile already
+// ended by its first segment, as dense tiles are.
 template <int TW, int TH, bool COUNT, bool SPLIT>
 __global__ void __launch_bounds__(TW * TH / 2, (TW * TH / 2 >= 128 ? 1024 / (TW * TH / 2) : 16))
     render_fwd_kernel(FwdArgs A) {
@@ -468,21 +470,28 @@ __global__ void __launch_bounds__(TW * TH / 2, (TW * TH / 2 >= 128 ? 1024 / (TW 
   if constexpr (SPLIT) {
     constexpr int TP = TW * TH;  // pixels per tile: the float4 pairs of a slot
     if (t >= A.n_tiles) {
-      // extra segment e: the split tile whose extra segments [w, w + m - 1) hold it
-      const uint32_t e = t - A.n_tiles;
-      if (e >= A.hdr->ctr[6]) return;
-      const uint32_t i = A.ext_owner[e];
-      const uint4 sp = A.split_list[i];
-      const uint32_t k = e - sp.w + 1;
-      fwd_tile<TW, TH, COUNT, true>(A, sp.x, sm, k * kSegLen, (k + 1) * kSegLen,
-                                    A.seg_buf + (size_t)(sp.y + k) * TP * 2, false, A.split_term + i, k);
+      // extra segments, from this CTA's first by the number of such CTAs: the
+      // split tile whose extra segments [w, w + m - 1) hold e
+      const uint32_t n_extra = A.hdr->ctr[6];
+      const uint32_t len = A.hdr->ctr[kCtrSegLen];
+      for (uint32_t e = t - A.n_tiles; e < n_extra; e += A.max_extra) {
+        const uint32_t i = A.ext_owner[e];
+        const uint4 sp = A.split_list[i];
+        const uint32_t k = e - sp.w + 1;
+        const size_t at = (size_t)(sp.y + k) * TP;
+        fwd_tile<TW, TH, COUNT, true>(A, sp.x, sm, k * len, (k + 1) * len, A.seg_c + at, A.seg_l + at, nullptr,
+                                      A.split_term + i, k);
+        __syncthreads();  // shared memory is free for the next segment
+      }
       return;
     }
     const uint32_t g = A.tile_order && order_dense(A.hdr, A.n_tiles, A.cap) ? A.tile_order[t] : t;
     const uint32_t i = A.tile_split[g];
-    if (i != 0xffffffffu)
-      fwd_tile<TW, TH, COUNT, true>(A, g, sm, 0, kSegLen, A.seg_buf + (size_t)A.split_list[i].y * TP * 2, false,
+    if (i != 0xffffffffu) {
+      const size_t at = (size_t)A.split_list[i].y * TP;
+      fwd_tile<TW, TH, COUNT, true>(A, g, sm, 0, A.hdr->ctr[kCtrSegLen], A.seg_c + at, A.seg_l + at, nullptr,
                                     A.split_term + i, 0);
+    }
     else
       fwd_tile<TW, TH, COUNT, true>(A, g, sm);
   } else {
@@ -492,26 +501,41 @@ __global__ void __launch_bounds__(TW * TH / 2, (TW * TH / 2 >= 128 ? 1024 / (TW 
 }
 
 
-// The plan of split lists: every tile whose list holds more than kSegLen
-// entries gets a split index i, m = ceil(n / kSegLen) consecutive slots of
-// segment state and m - 1 extra segments (CTAs of the split grids), in the
-// order the atomics hand them out; tile_split, slot_owner and ext_owner map
-// tiles, slots and extra segments to i.  The counters (header ctr[4..6]) are
-// zeroed before the launch.
+// The plan of split lists: every tile whose list holds more than kSplitMin
+// entries gets a split index i, m = ceil(n / len) consecutive slots of
+// segment state and m - 1 extra segments, in the order the atomics hand them
+// out; tile_split, slot_owner and ext_owner map tiles, slots and extra
+// segments to i.  The counters (header ctr[4..6]) are zeroed before the
+// launch.
+//
+// A segment is walked by one CTA (a warp per 8x8 block), entry after entry:
+// its time is its length times the latency of an entry, some 0.2 us forward
+// and 0.4 us backward when few segments share an SM, so short segments win
+// (two tiles of 29,000 entries and two of 7,700 in a sparse 1600x1060 view:
+// forward 385 + resume 279 + backward 589 us with 2048 entries, 157 + 75 +
+// 224 with 512, 106 + 23 + 157 with 128).  The length is the
+// shortest for which the slots hold every segment: the long lists' sort
+// chunks (n_long, of kSortChunk entries) bound their number, and seg_safe
+// is one that always does.
 __global__ void __launch_bounds__(256) split_plan_kernel(const uint32_t* __restrict__ tstart, uint32_t NT,
                                                          uint4* __restrict__ split_list,
                                                          uint32_t* __restrict__ tile_split,
                                                          uint32_t* __restrict__ slot_owner,
                                                          uint32_t* __restrict__ ext_owner,
-                                                         uint32_t* __restrict__ split_term, uint32_t max_split,
+                                                         uint32_t* __restrict__ split_term, uint32_t seg_min,
+                                                         uint32_t seg_safe, uint32_t max_split,
                                                          uint32_t max_slots, uint32_t max_extra, Header* hdr) {
   wait_prior_grid();
   if (hdr->status != 0) return;
+  uint32_t seg_len = seg_min;
+  while (seg_len < seg_safe && (uint64_t)hdr->n_long * (seg_len < kSortChunk ? kSortChunk / seg_len : 1u) > max_slots)
+    seg_len *= 2;
+  if (blockIdx.x == 0 && threadIdx.x == 0) hdr->ctr[kCtrSegLen] = seg_len;
   for (uint32_t g = blockIdx.x * 256 + threadIdx.x; g < NT; g += gridDim.x * 256) {
     const uint32_t n = tstart[g + 1] - tstart[g];
     uint32_t split = 0xffffffffu;
-    if (n > kSegLen) {
-      const uint32_t m = (n + kSegLen - 1) / kSegLen;
+    if (n > kSplitMin) {
+      const uint32_t m = (n + seg_len - 1) / seg_len;
       const uint32_t i = atomicAdd(&hdr->ctr[4], 1u);
       const uint32_t b = atomicAdd(&hdr->ctr[5], m);
       const uint32_t e = atomicAdd(&hdr->ctr[6], m - 1);
@@ -563,54 +587,105 @@ __global__ void __launch_bounds__(TW * TH / 2, (TW * TH / 2 >= 128 ? 1024 / (TW 
 // (the local walk stopped, or T T_k < T_min) is where the pixel's walk ends,
 // and that segment is walked again from the pixel's true T.
 //
-// Pass 1 (one CTA per split tile, a thread per pixel): the over operator up
-// to k*.  Slot k < k* gets the colour segment k adds (absolute) and T at its
-// end; slot k* gets the pixel's T and last contributor at its start and a
-// "walk again" mark; slot 0 records k* (m when the walk never ends early)
-// and the last contributor.
-template <int TW, int TH>
-__global__ void __launch_bounds__(TW * TH) split_join_kernel(FwdArgs A) {
-  wait_prior_grid();
-  constexpr int TP = TW * TH;
-  if (A.hdr->status != 0) return;
-  if (blockIdx.x >= A.hdr->ctr[4]) return;
-  const uint4 sp = A.split_list[blockIdx.x];
-  const uint32_t m = sp.z;
-  float4* my = A.seg_buf + (size_t)sp.y * TP * 2 + 2 * threadIdx.x;  // slot k: my[2 k TP], my[2 k TP + 1]
-  const CfgDev& cfg = A.cfg;
-  const float4 s0 = my[0], s1 = my[1];
-  float T = s0.w;
-  uint32_t last = __float_as_uint(s1.x);
-  bool done = __float_as_uint(s1.y) != 0u;  // ended in the first segment (exact), or outside the image
-  uint32_t kstar = m;
-  my[1] = make_float4(s1.x, 0.0f, 0.0f, 0.0f);
-  for (uint32_t k = 1; k < m; ++k) {
-    float4* mk = my + (size_t)2 * k * TP;
-    const float4 a0 = mk[0], a1 = mk[1];
-    if (kstar < m || done) {  // after the walk ended: the segment adds nothing
-      mk[0] = make_float4(0.0f, 0.0f, 0.0f, T);
-      mk[1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      continue;
-    }
-    const float Tk = __fmul_rn(T, a0.w);
-    if (__float_as_uint(a1.y) != 0u || Tk < cfg.tmin) {
-      kstar = k;
-      mk[0] = make_float4(0.0f, 0.0f, 0.0f, T);
-      mk[1] = make_float4(__uint_as_float(last), __uint_as_float(1u), 0.0f, 0.0f);
-      continue;
-    }
-    mk[0] = make_float4(__fmul_rn(T, a0.x), __fmul_rn(T, a0.y), __fmul_rn(T, a0.z), Tk);
-    mk[1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    T = Tk;
-    const uint32_t lk = __float_as_uint(a1.x);
-    last = lk ? lk : last;
-  }
-  my[1] = make_float4(__uint_as_float(last), 0.0f, __uint_as_float(kstar), 0.0f);
+// Passes 1 and 3 give a CTA 32 pixels of a split tile, a pixel per lane, and
+// each of its kJoinW warps an equal run of the tile's segments: a walk over
+// all segments by one thread per pixel is bound by the latency of its loads
+// (226 segments: 50 and 112 us for the two passes; 14 and 12 us so).
+constexpr int kJoinW = 8;
+// warp w's segments [k0, k1) of m, from segment `first`
+__device__ __forceinline__ void join_share(uint32_t first, uint32_t m, int w, uint32_t& k0, uint32_t& k1) {
+  const uint32_t n = m > first ? m - first : 0u, per = (n + kJoinW - 1) / kJoinW;
+  k0 = min(m, first + w * per);
+  k1 = min(m, k0 + per);
 }
 
-// Pass 2 (one CTA per slot): the segments that pass 1 marked are walked
-// again, with the forward blend's own tile walk, only for the marked pixels,
-// from their true T (colour from zero); all the segments run at once.
+// Pass 1: the over operator up to k*.  Slot k < k* gets the colour segment k
+// adds (absolute) and T at its end; slot k* gets the pixel's T and last
+// contributor at its start.  The pixel's seg_end is k* | kSegEnded ("walk
+// again") where the walk ends in a later segment, else the last segment that
+// adds anything (0 where the walk ended in the first, exact one); slot 0 gets
+// the last contributor up to there.  The slots after seg_end are not read
+// again.  Each warp first folds its run (T's product, last contributor,
+// whether a segment ended the pixel), and after a barrier walks it from the
+// T that the runs before it leave, unless the pixel ended there.
+template <int TW, int TH>
+__global__ void __launch_bounds__(32 * kJoinW) split_join_kernel(FwdArgs A) {
+  wait_prior_grid();
+  constexpr int TP = TW * TH, CPT = TP / 32;  // CTAs' shares per tile
+  __shared__ float s_T[kJoinW][32];
+  __shared__ uint32_t s_last[kJoinW][32], s_end[32], s_fin[32];
+  if (A.hdr->status != 0) return;
+  const CfgDev& cfg = A.cfg;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t n_items = A.hdr->ctr[4] * CPT;
+  for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
+    const uint4 sp = A.split_list[it / CPT];
+    const uint32_t m = sp.z, px = (it % CPT) * 32 + lane;
+    float4* my = A.seg_c + (size_t)sp.y * TP + px;  // slot k: my[k TP], my_l[k TP]
+    uint32_t* my_l = A.seg_l + (size_t)sp.y * TP + px;
+    const float T0 = my[0].w;
+    const uint32_t l0 = my_l[0];
+    uint32_t k0, k1;
+    join_share(1, m, w, k0, k1);
+    float T = 1.0f;
+    uint32_t last = 0;  // with kSegEnded where a segment ended the pixel
+#pragma unroll 4
+    for (uint32_t k = k0; k < k1; ++k) {
+      const float a = my[(size_t)k * TP].w;
+      const uint32_t l = my_l[(size_t)k * TP];
+      T = __fmul_rn(T, a);
+      last = (last & kSegEnded) | (l & kSegEnded) | ((l & ~kSegEnded) ? l & ~kSegEnded : last & ~kSegEnded);
+    }
+    s_T[w][lane] = T;
+    s_last[w][lane] = last;
+    if (w == 0) s_end[lane] = (l0 & kSegEnded) ? 0u : m - 1;  // ended in the first segment, or outside the image
+    __syncthreads();
+    float T1 = T0;  // at the start of this run
+    last = l0 & ~kSegEnded;
+    bool on = (l0 & kSegEnded) == 0u;
+    for (int h = 0; h < w; ++h) {  // the runs before this one
+      T1 = __fmul_rn(T1, s_T[h][lane]);
+      const uint32_t l = s_last[h][lane];
+      on = on && !(l & kSegEnded) && T1 >= cfg.tmin;
+      last = (l & ~kSegEnded) ? l & ~kSegEnded : last;
+    }
+    // T at the end of segment k is T1 times the run's product up to k: the
+    // product of the fold, so that the runs agree on where the walk ends
+    T = 1.0f;
+#pragma unroll 4
+    for (uint32_t k = k0; k < k1; ++k) {
+      const float4 a = my[(size_t)k * TP];
+      const uint32_t l = my_l[(size_t)k * TP];
+      const float Ts = __fmul_rn(T1, T);  // at its start
+      T = __fmul_rn(T, a.w);
+      const float Tk = __fmul_rn(T1, T);
+      if (!on) continue;
+      if ((l & kSegEnded) || Tk < cfg.tmin) {
+        on = false;
+        s_end[lane] = k | kSegEnded;  // one warp's: no later run goes on
+        my[(size_t)k * TP].w = Ts;
+        my_l[(size_t)k * TP] = last;
+        continue;
+      }
+      my[(size_t)k * TP] = make_float4(__fmul_rn(Ts, a.x), __fmul_rn(Ts, a.y), __fmul_rn(Ts, a.z), Tk);
+      last = l ? l : last;
+    }
+    // the last contributor over the whole walk: of the last run that goes on
+    if (w == kJoinW - 1 && on) s_fin[lane] = last;
+    __syncthreads();
+    if (w == 0) {
+      const uint32_t end = s_end[lane];
+      A.seg_end[(size_t)(it / CPT) * TP + px] = end;
+      // with a walk that ends in a later segment, that segment's own counts
+      my_l[0] = end == m - 1 ? s_fin[lane] : l0 & ~kSegEnded;
+    }
+    __syncthreads();  // shared memory is free for the next share
+  }
+}
+
+// Pass 2 (CTAs looping over the slots): the segments that pass 1 marked are
+// walked again, with the forward blend's own tile walk, only for the marked
+// pixels, from their true T (colour from zero); all the segments run at once.
 template <int TW, int TH>
 __global__ void __launch_bounds__(TW * TH / 2, (TW * TH / 2 >= 128 ? 1024 / (TW * TH / 2) : 16))
     split_resume_kernel(FwdArgs A) {
@@ -618,70 +693,98 @@ __global__ void __launch_bounds__(TW * TH / 2, (TW * TH / 2 >= 128 ? 1024 / (TW 
   constexpr int TP = TW * TH;
   __shared__ FwdSmem<TW, TH> sm;
   if (A.hdr->status != 0) return;
-  const uint32_t s = blockIdx.x;
-  if (s >= A.hdr->ctr[5]) return;  // unused
-  const uint4 sp = A.split_list[A.slot_owner[s]];
-  const uint32_t k = s - sp.y;
-  if (k == 0) return;  // the first segment is exact
-  fwd_tile<TW, TH, false, true>(A, sp.x, sm, k * kSegLen, (k + 1) * kSegLen, A.seg_buf + (size_t)s * TP * 2, true);
+  const uint32_t n = A.hdr->ctr[5], len = A.hdr->ctr[kCtrSegLen];
+  for (uint32_t s = blockIdx.x; s < n; s += gridDim.x) {
+    const uint32_t i = A.slot_owner[s];
+    const uint4 sp = A.split_list[i];
+    const uint32_t k = s - sp.y;
+    if (k == 0) continue;  // the first segment is exact
+    const uint32_t* end = A.seg_end + (size_t)i * TP;
+    const bool any = end[threadIdx.x] == (k | kSegEnded) || end[threadIdx.x + TP / 2] == (k | kSegEnded);
+    if (__syncthreads_or(any) == 0) continue;  // no pixel ends here; also: shared memory is free for this segment
+    const size_t at = (size_t)s * TP;
+    fwd_tile<TW, TH, false, true>(A, sp.x, sm, k * len, (k + 1) * len, A.seg_c + at, A.seg_l + at, end, nullptr, k);
+  }
 }
 
-// Pass 3 (one CTA per split tile, a thread per pixel): the pixel's colour,
-// final T and last contributor, written to the image; and, for the
-// backward, each segment's T at its end and the colour behind it
-// (everything after it and the background), normalised by that T.
+// Pass 3: the pixel's colour, final T and last contributor, written to the
+// image; and, for the backward, each segment's T at its end and the colour
+// behind it (everything after it and the background), normalised by that T,
+// up to the segment the walk ends in (the backward reads no later one).
+// Each warp sums its run's colours, and then walks it back from the sum of
+// the later runs.
 template <int TW, int TH>
-__global__ void __launch_bounds__(TW * TH) split_finish_kernel(FwdArgs A) {
+__global__ void __launch_bounds__(32 * kJoinW) split_finish_kernel(FwdArgs A) {
   wait_prior_grid();
-  constexpr int TP = TW * TH;
+  constexpr int TP = TW * TH, CPT = TP / 32;
   __shared__ int s_v;
+  __shared__ float4 s_c[kJoinW][32];
   if (A.hdr->status != 0) return;
-  if (blockIdx.x >= A.hdr->ctr[4]) return;
-  const uint4 sp = A.split_list[blockIdx.x];
-  const uint32_t g = sp.x, m = sp.z;
-  if (threadIdx.x < 32) {
-    const int vi = find_view_warp(A.views, A.V, g);
-    if (threadIdx.x == 0) s_v = vi;
-  }
-  __syncthreads();
-  const ViewDev& v = A.views[s_v];
   const CfgDev& cfg = A.cfg;
-  float4* my = A.seg_buf + (size_t)sp.y * TP * 2 + 2 * threadIdx.x;
-  const float4 h1 = my[1];
-  uint32_t last = __float_as_uint(h1.x);
-  const uint32_t kstar = __float_as_uint(h1.z);
-  float C0 = 0.0f, C1 = 0.0f, C2 = 0.0f, T = 1.0f;
-  const uint32_t kend = kstar < m ? kstar : m - 1;  // the segment the walk ends in
-  for (uint32_t k = 0; k <= kend; ++k) {
-    const float4 a0 = my[(size_t)2 * k * TP];
-    C0 += a0.x;
-    C1 += a0.y;
-    C2 += a0.z;
-    T = a0.w;
-  }
-  if (kstar < m) last = __float_as_uint(my[(size_t)2 * kstar * TP + 1].x);
-  const uint32_t lt = g - v.tile_off;
-  const int tx = lt % v.tiles_x, ty = lt / v.tiles_x;
-  const int x = tx * TW + (int)(threadIdx.x % TW), y = ty * TH + (int)(threadIdx.x / TW);
-  if (x < v.W && y < v.H) {
-    const size_t plane = (size_t)v.W * v.H, pix = (size_t)y * v.W + x;
-    float* img = A.image + (size_t)v.pix_off * 3;
-    img[pix] = fmaf(T, cfg.bg[0], C0);
-    img[plane + pix] = fmaf(T, cfg.bg[1], C1);
-    img[2 * plane + pix] = fmaf(T, cfg.bg[2], C2);
-    A.Tfin[v.pix_off + pix] = T;
-    A.lastc[v.pix_off + pix] = last;
-  }
-  float b0 = T * cfg.bg[0], b1 = T * cfg.bg[1], b2 = T * cfg.bg[2];
-  for (int k = (int)m - 1; k >= 0; --k) {
-    float4* mk = my + (size_t)2 * k * TP;
-    float4 a0 = make_float4(0.0f, 0.0f, 0.0f, T);  // after the walk ended: nothing added, T final
-    if ((uint32_t)k <= kend) a0 = mk[0];
-    const float inv = a0.w > 0.0f ? 1.0f / a0.w : 0.0f;
-    mk[1] = make_float4(b0 * inv, b1 * inv, b2 * inv, a0.w);
-    b0 += a0.x;
-    b1 += a0.y;
-    b2 += a0.z;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t n_items = A.hdr->ctr[4] * CPT;
+  for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
+    const uint4 sp = A.split_list[it / CPT];
+    const uint32_t g = sp.x, px = (it % CPT) * 32 + lane;
+    if (w == 0) {
+      const int vi = find_view_warp(A.views, A.V, g);
+      if (lane == 0) s_v = vi;
+    }
+    float4* my = A.seg_c + (size_t)sp.y * TP + px;
+    const uint32_t* my_l = A.seg_l + (size_t)sp.y * TP + px;
+    const uint32_t end = A.seg_end[(size_t)(it / CPT) * TP + px];
+    const uint32_t kend = end & ~kSegEnded;  // the last segment that adds anything
+    uint32_t k0, k1;
+    join_share(0, sp.z, w, k0, k1);
+    k1 = min(k1, kend + 1);
+    float C0 = 0.0f, C1 = 0.0f, C2 = 0.0f;
+#pragma unroll 4
+    for (uint32_t k = k0; k < k1; ++k) {
+      const float4 a = my[(size_t)k * TP];
+      C0 += a.x;
+      C1 += a.y;
+      C2 += a.z;
+    }
+    const float T = my[(size_t)kend * TP].w;
+    s_c[w][lane] = make_float4(C0, C1, C2, 0.0f);
+    __syncthreads();
+    if (w == 0) {
+      const ViewDev& v = A.views[s_v];
+      const uint32_t lt = g - v.tile_off;
+      const int tx = lt % v.tiles_x, ty = lt / v.tiles_x;
+      const int x = tx * TW + (int)(px % TW), y = ty * TH + (int)(px / TW);
+      if (x < v.W && y < v.H) {
+        for (int h = 1; h < kJoinW; ++h) {
+          C0 += s_c[h][lane].x;
+          C1 += s_c[h][lane].y;
+          C2 += s_c[h][lane].z;
+        }
+        const size_t plane = (size_t)v.W * v.H, pix = (size_t)y * v.W + x;
+        float* img = A.image + (size_t)v.pix_off * 3;
+        img[pix] = fmaf(T, cfg.bg[0], C0);
+        img[plane + pix] = fmaf(T, cfg.bg[1], C1);
+        img[2 * plane + pix] = fmaf(T, cfg.bg[2], C2);
+        A.Tfin[v.pix_off + pix] = T;
+        A.lastc[v.pix_off + pix] = my_l[(end & kSegEnded) ? (size_t)kend * TP : 0];
+      }
+    }
+    float b0 = T * cfg.bg[0], b1 = T * cfg.bg[1], b2 = T * cfg.bg[2];
+    for (int h = kJoinW - 1; h > w; --h) {
+      b0 += s_c[h][lane].x;
+      b1 += s_c[h][lane].y;
+      b2 += s_c[h][lane].z;
+    }
+#pragma unroll 4
+    for (int k = (int)k1 - 1; k >= (int)k0; --k) {
+      float4* mk = my + (size_t)k * TP;
+      const float4 a = *mk;
+      const float inv = a.w > 0.0f ? 1.0f / a.w : 0.0f;
+      *mk = make_float4(b0 * inv, b1 * inv, b2 * inv, a.w);
+      b0 += a.x;
+      b1 += a.y;
+      b2 += a.z;
+    }
+    __syncthreads();  // shared memory is free for the next share
   }
 }
 
@@ -771,8 +874,8 @@ struct BwdArgs {
   const uint4* split_list;
   const uint32_t* tile_split;
   const uint32_t* ext_owner;
-  const float4* seg_buf;
-  uint32_t max_extra;
+  const float4* seg_c;
+  uint32_t max_extra;  // CTAs of extra segments (per 8x8 block), each looping
 };
 
 // One 8x8 block wb of tile g, by one warp.  With SPLIT and a slot, only the
@@ -825,12 +928,21 @@ __device__ __forceinline__ void bwd_block(const BwdArgs& A, uint32_t g, int wb, 
     }
   }
   if constexpr (SPLIT) {
-    if (slot) {  // the segment's end: T and the normalised colour behind it
-      const float4 s0 = slot[2 * (ly * TW + lx) + 1], s1 = slot[2 * ((ly + 4) * TW + lx) + 1];
-      T = make_float2(s0.w, s1.w);
-      B0 = make_float2(s0.x, s1.x);
-      B1 = make_float2(s0.y, s1.y);
-      B2 = make_float2(s0.z, s1.z);
+    // the segment's end: T and the normalised colour behind it, for the pixels
+    // whose walk reaches the segment (the others use no entry of it)
+    if (slot && last0 > wbeg) {
+      const float4 s0 = slot[ly * TW + lx];
+      T.x = s0.w;
+      B0.x = s0.x;
+      B1.x = s0.y;
+      B2.x = s0.z;
+    }
+    if (slot && last1 > wbeg) {
+      const float4 s1 = slot[(ly + 4) * TW + lx];
+      T.y = s1.w;
+      B0.y = s1.x;
+      B1.y = s1.y;
+      B2.y = s1.z;
     }
   }
   uint32_t wlast = __reduce_max_sync(kFull, max(last0, last1));
@@ -939,8 +1051,8 @@ __device__ __forceinline__ void bwd_block(const BwdArgs& A, uint32_t g, int wb, 
 }
 
 // The grid form: one single-warp CTA per 8x8 block.  With SPLIT the grid
-// first holds the blocks of A.max_extra extra segments (those the plan did
-// not assign exit), and a split tile's own blocks walk its first segment.
+// first holds the blocks of A.max_extra CTAs for the extra segments, each
+// walking every max_extra-th, and a split tile's own blocks walk its first.
 template <int TW, int TH, bool SPLIT>
 __global__ void __launch_bounds__(32, 32)  // 64 registers: 32 one-warp CTAs per SM
     render_bwd_kernel(BwdArgs A) {
@@ -953,18 +1065,21 @@ __global__ void __launch_bounds__(32, 32)  // 64 registers: 32 one-warp CTAs per
   if constexpr (SPLIT) {
     constexpr int TP = TW * TH;
     if (t < A.max_extra) {
-      if (t >= A.hdr->ctr[6]) return;
-      const uint4 sp = A.split_list[A.ext_owner[t]];
-      const uint32_t k = t - sp.w + 1;
-      bwd_block<TW, TH, true>(A, sp.x, wb, sm, k * kSegLen, (k + 1) * kSegLen,
-                              A.seg_buf + (size_t)(sp.y + k) * TP * 2);
+      const uint32_t n_extra = A.hdr->ctr[6], len = A.hdr->ctr[kCtrSegLen];
+      for (uint32_t e = t; e < n_extra; e += A.max_extra) {
+        const uint4 sp = A.split_list[A.ext_owner[e]];
+        const uint32_t k = e - sp.w + 1;
+        bwd_block<TW, TH, true>(A, sp.x, wb, sm, k * len, (k + 1) * len,
+                                A.seg_c + (size_t)(sp.y + k) * TP);
+        __syncwarp();
+      }
       return;
     }
     t -= A.max_extra;
     const uint32_t g = A.tile_order && order_dense(A.hdr, A.n_tiles, A.cap) ? A.tile_order[t] : t;
     const uint32_t i = A.tile_split[g];
     if (i != 0xffffffffu)
-      bwd_block<TW, TH, true>(A, g, wb, sm, 0, kSegLen, A.seg_buf + (size_t)A.split_list[i].y * TP * 2);
+      bwd_block<TW, TH, true>(A, g, wb, sm, 0, A.hdr->ctr[kCtrSegLen], A.seg_c + (size_t)A.split_list[i].y * TP);
     else
       bwd_block<TW, TH, true>(A, g, wb, sm);
   } else {
@@ -1049,7 +1164,12 @@ cudaError_t fwd_launch(const FwdArgs& args, const Layout& L, bool persistent, cu
 }
 
 // Split lists: the plan (after zeroing its counters), the grid of extra
-// segments and tiles, and the merge of the split tiles.
+// segments and tiles, and the merge of the split tiles.  The grids over
+// segments, slots and split tiles are sized by the capacity's bounds, which
+// the lists rarely come near, up to a few CTAs per SM; beyond that they loop.
+constexpr uint32_t kSplitGrid = 152 * 8;
+inline uint32_t split_grid(uint32_t n) { return n < kSplitGrid ? n : kSplitGrid; }
+
 template <int TW, int TH>
 cudaError_t fwd_split(const FwdArgs& args, const Layout& L, char* ws, cudaStream_t st) {
   constexpr int NT = TW * TH / 2;
@@ -1060,15 +1180,17 @@ cudaError_t fwd_split(const FwdArgs& args, const Layout& L, char* ws, cudaStream
   e = launch_dependent(split_plan_kernel, dim3(pb < 1024 ? pb : 1024), dim3(256), 0, st,
                        (const uint32_t*)(ws + L.tstart), L.NT, (uint4*)(ws + L.split_list),
                        (uint32_t*)(ws + L.tile_slot), (uint32_t*)(ws + L.slot_owner), (uint32_t*)(ws + L.ext_owner),
-                       (uint32_t*)(ws + L.split_term), L.seg_max_split, L.seg_slots, L.seg_max_extra, hdr);
+                       (uint32_t*)(ws + L.split_term),
+                       (uint32_t)(FwdSmem<TW, TH>::BS > kSegMin ? FwdSmem<TW, TH>::BS : kSegMin), L.seg_safe, L.seg_max_split, L.seg_slots, L.seg_max_extra, hdr);
   if (e != cudaSuccess) return e;
-  e = launch_dependent(render_fwd_kernel<TW, TH, false, true>, dim3(L.seg_max_extra + L.NT), dim3(NT), 0, st, args);
+  e = launch_dependent(render_fwd_kernel<TW, TH, false, true>, dim3(args.max_extra + L.NT), dim3(NT), 0, st, args);
   if (e != cudaSuccess) return e;
-  e = launch_dependent(split_join_kernel<TW, TH>, dim3(L.seg_max_split), dim3(TW * TH), 0, st, args);
+  const dim3 shares(split_grid(L.seg_max_split * (TW * TH / 32)));
+  e = launch_dependent(split_join_kernel<TW, TH>, shares, dim3(32 * kJoinW), 0, st, args);
   if (e != cudaSuccess) return e;
-  e = launch_dependent(split_resume_kernel<TW, TH>, dim3(L.seg_slots), dim3(NT), 0, st, args);
+  e = launch_dependent(split_resume_kernel<TW, TH>, dim3(args.max_slots), dim3(NT), 0, st, args);
   if (e != cudaSuccess) return e;
-  return launch_dependent(split_finish_kernel<TW, TH>, dim3(L.seg_max_split), dim3(TW * TH), 0, st, args);
+  return launch_dependent(split_finish_kernel<TW, TH>, shares, dim3(32 * kJoinW), 0, st, args);
 }
 
 template <int TW, int TH>
@@ -1098,8 +1220,11 @@ cudaError_t fwd_t(const Layout& L, const CfgDev& cfg, char* ws, float* image, cu
   a.slot_owner = split ? (const uint32_t*)(ws + L.slot_owner) : nullptr;
   a.ext_owner = split ? (const uint32_t*)(ws + L.ext_owner) : nullptr;
   a.split_term = split ? (uint32_t*)(ws + L.split_term) : nullptr;
-  a.seg_buf = split ? (float4*)(ws + L.seg_buf) : nullptr;
-  a.max_extra = split ? L.seg_max_extra : 0;
+  a.seg_c = split ? (float4*)(ws + L.seg_c) : nullptr;
+  a.seg_l = split ? (uint32_t*)(ws + L.seg_l) : nullptr;
+  a.seg_end = split ? (uint32_t*)(ws + L.seg_end) : nullptr;
+  a.max_extra = split ? split_grid(L.seg_max_extra) : 0;
+  a.max_slots = split ? split_grid(L.seg_slots) : 0;
   if (split) return fwd_split<TW, TH>(a, L, ws, st);
   const bool persistent = (cfg.flags & 8) != 0;
   return count ? fwd_launch<TW, TH, true>(a, L, persistent, st) : fwd_launch<TW, TH, false>(a, L, persistent, st);
@@ -1130,10 +1255,10 @@ cudaError_t bwd_t(const Layout& L, const CfgDev& cfg, char* ws, const float* dL,
   a.split_list = split ? (const uint4*)(ws + L.split_list) : nullptr;
   a.tile_split = split ? (const uint32_t*)(ws + L.tile_slot) : nullptr;
   a.ext_owner = split ? (const uint32_t*)(ws + L.ext_owner) : nullptr;
-  a.seg_buf = split ? (const float4*)(ws + L.seg_buf) : nullptr;
-  a.max_extra = split ? L.seg_max_extra : 0;
+  a.seg_c = split ? (const float4*)(ws + L.seg_c) : nullptr;
+  a.max_extra = split ? split_grid(L.seg_max_extra) : 0;
   if (split) {
-    launch_dependent(render_bwd_kernel<TW, TH, true>, dim3((L.seg_max_extra + L.NT) * (TW * TH / 64)), dim3(32), 0,
+    launch_dependent(render_bwd_kernel<TW, TH, true>, dim3((a.max_extra + L.NT) * (TW * TH / 64)), dim3(32), 0,
                      st, a);
     return cudaGetLastError();
   }

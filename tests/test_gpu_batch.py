@@ -11,6 +11,7 @@ import torch
 from paper_2510_03312_gb300 import autotune as A
 from paper_2510_03312_gb300 import raster
 from paper_2510_03312_gb300 import scenes as S
+from paper_2510_03312_gb300 import ubs as U
 
 pytestmark = pytest.mark.gpu
 
@@ -177,3 +178,37 @@ def test_dense_lists_over_many_tiles_match_views_alone():
         torch.cuda.synchronize()
         assert torch.equal(imgp, r.image)
         assert _close(gp, g)
+
+
+@pytest.mark.parametrize("tile", [(8, 8), (16, 16), (16, 32), (32, 32)])
+@pytest.mark.parametrize("n,cap", [(2049, None), (2304, None), (9000, None), (9000, 3_000_000)])
+def test_split_segments_at_their_edges(tile, n, cap):
+    """One tile's list one entry over the split length, at a multiple of the
+    shortest segment and many segments long, with a workspace that holds the
+    shortest segments and (a capacity far above the lists) one that holds
+    fewer, per tile shape: the image within 1e-5 of the unsplit form's and
+    the gradients within 1e-3 of their plane's largest, the bounds of the
+    oracle comparisons."""
+    rng = np.random.default_rng(n)
+    sc = S.make_scene(n, 3, n, scale_range=(0.02, 0.05), rng=rng)
+    sc.plane("mean_x")[:] = (0.0005 * rng.uniform(-1.0, 1.0, (3, n))).astype(np.float32)
+    # the shorter lists' pixel stays above T_min to their end, the long one's ends in some middle segment
+    op = rng.choice([0.0043, 0.01], n, p=[0.98, 0.02]) if n < 9000 else rng.choice([0.005, 0.02, 0.1], n)
+    sc.plane("opacity")[:] = op.astype(np.float32)
+    v = S.make_view(np.eye(3), np.array([0.0, 0.0, 4.0]), 75, 71)  # the stack's mean at a pixel's centre
+    got = {}
+    for split in (False, True):
+        r = raster.Rasterizer([raster.DeviceScene.from_scene(sc, device="cuda")], [v],
+                              S.RasterConfig(tile_w=tile[0], tile_h=tile[1], split_lists=split), capacity=cap,
+                              device="cuda")
+        for _ in range(2):  # the second on the segment state the first left
+            r.preprocess()
+            r.bin_sort()
+            img = r.render_fwd().clone()
+        st = r.status()
+        assert st.status == 0 and torch.diff(r.export(U.EXPORT_TILE_START)).max() > 2048
+        dL = torch.sin(torch.arange(img.numel(), device="cuda")) / img.numel()
+        got[split] = img, r.backward(dL)[0].clone()
+    assert (got[True][0] - got[False][0]).abs().max() <= 1e-5
+    worst = ((got[True][1] - got[False][1]).abs().amax(1) / got[False][1].abs().amax(1).clamp(min=1e-30)).max()
+    assert worst <= 1e-3, float(worst)
