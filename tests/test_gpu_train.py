@@ -211,3 +211,25 @@ def test_binding_rejects_bad_tensors_before_launching(dev):
     ds.params = ds.params.clone()  # the problem still holds the old pointers
     with pytest.raises(ValueError, match="replaced"):
         r.preprocess()
+
+
+@pytest.mark.parametrize("sizes", [[(128, 16)], [(129, 17)], [(127, 15)], [(256, 20)], [(31, 200)], [(5, 97)],
+                                   [(133, 33), (1, 1), (257, 64)]])
+def test_image_loss_at_strip_edges(dev, sizes):
+    """The loss and its gradient where a strip of output columns or rows just
+    fills, overflows or falls short, and narrow, tall images (more rows than
+    block sums would allow in short strips), against the float64 reference,
+    with the bounds of the larger cases."""
+    rng = np.random.default_rng(len(sizes) + sizes[0][0])
+    from paper_2510_03312_gb300 import train as TR
+    xs = [rng.random((3, h, w)).astype(np.float32) for w, h in sizes]
+    ys = [np.clip(x + 0.15 * rng.standard_normal(x.shape), 0, 1).astype(np.float32) for x in xs]
+    loss_fn = TR.ImageLoss([_V(w, h) for w, h in sizes], device=dev)
+    dL = torch.empty(sum(3 * w * h for w, h in sizes), device=dev)
+    out = loss_fn(_pack(xs, dev), _pack(ys, dev), dL).cpu().numpy()
+    ref, per, grads = T.image_loss(xs, ys, TR.LAMBDA_SSIM)
+    assert out[0] == pytest.approx(ref, rel=2e-5, abs=1e-7)
+    assert np.allclose(out[1:], per, rtol=2e-5, atol=1e-7)
+    gmax = max(np.abs(g).max() for g in grads)
+    for a, b in zip(_unpack(dL.cpu().numpy(), sizes), grads):
+        assert np.abs(a - b).max() <= 1e-4 * gmax + 1e-3 * np.abs(b).max()
