@@ -233,3 +233,35 @@ def test_image_loss_at_strip_edges(dev, sizes):
     gmax = max(np.abs(g).max() for g in grads)
     for a, b in zip(_unpack(dL.cpu().numpy(), sizes), grads):
         assert np.abs(a - b).max() <= 1e-4 * gmax + 1e-3 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("P", [1, 2, 3, 5, 6, 1023, 4097])
+def test_adam_words_across_planes(dev, P):
+    """Four-element words that straddle planes (P not a multiple of four, down
+    to planes shorter than a word): against the oracle (up to about a thousand
+    parameters a plane, the size its bounds are made for), and bit for bit
+    against the same step on buffers off the 16-byte boundary, which goes
+    element by element."""
+    import ctypes
+
+    from paper_2510_03312_gb300 import train as TR
+    from paper_2510_03312_gb300 import ubs as U
+    if P < 2000:
+        test_adam_step_matches_oracle(dev, P)
+    table = TR.plane_table(6, S.ROT_SKEW1, TR.TrainConfig())
+    K = len(table)
+    planes = (U.ubs_adam_plane * K)()
+    for k, (lr, a, l1, row) in enumerate(table):
+        planes[k].lr, planes[k].activation, planes[k].l1_weight, planes[k].noise_row = lr, a, l1, row
+    g = torch.Generator(device=dev).manual_seed(P)
+    src = [torch.randn(K * P, generator=g, device=dev) * s for s in (0.5, 1.0, 1e-2, 1e-3)] + \
+          [torch.rand(K * P, generator=g, device=dev) * 1e-5, torch.randn(3 * P, generator=g, device=dev) * 1e-3]
+    out = []
+    for off in (0, 1):
+        raw, act, grad, m, v, noise = [torch.cat([torch.zeros(off, device=dev), s])[off:] for s in src]
+        st = U.ubs_adam_step(K, P, planes, U.ubs_adam_config(0.9, 0.999, 1e-15, 7, 1.0), raw.data_ptr(), act.data_ptr(),
+                             grad.data_ptr(), m.data_ptr(), v.data_ptr(), noise.data_ptr(),
+                             ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert st == U.UBS_OK
+        out.append((raw, act, m, v))
+    assert all(torch.equal(a, b) for a, b in zip(*out))
