@@ -1,8 +1,9 @@
 // prim_backward.cu -- G2: chain the per-record screen gradients back to the
 // primitive parameters (math in prim_backward.cuh).
 //
-// One thread per primitive (scenes with one view: every primitive; with
-// several: the list of primitives some view sees, built by preprocess); it
+// One thread per primitive (scenes with one view: every primitive for N = 3,
+// the drawn ones of its CTA's range for N > 3; with several: the list of
+// primitives some view sees, built by preprocess); it
 // rebuilds the view-independent quantities once, walks its visible views
 // accumulating in registers, and writes every parameter gradient once: no
 // atomics and a deterministic sum over views.
@@ -79,6 +80,98 @@ __global__ void __launch_bounds__(128, C == 0 ? 7 : 1) prim_backward_kernel(Scen
   }
 }
 
+
+// Scenes with query dimensions and one view: one CTA per kPbPrims consecutive
+// primitives.  It lists those the view draws (their visibility bits) in shared
+// memory and gives each thread listed ones, whose parameters lie close
+// together; then it writes zero gradients for the others (unless
+// accumulating).  The query culls most records (7% drawn), on which a thread
+// per primitive spent its loads and arithmetic all the same (200K N=6
+// primitives: 40 us; 17 us so).  Scenes with several views draw most primitives
+// in some view: there the list of the whole scene (prim_backward_listed_kernel)
+// balances better (16 views of 500K N=6 primitives: 11 + 98 us, this form 144).
+constexpr int kPbThreads = 128;
+constexpr int kPbPrims = 512, kPbWords = kPbPrims / 32;
+template <int C>
+__global__ void __launch_bounds__(kPbThreads, C == 3 ? 4 : 1) prim_backward_drawn_kernel(
+    SceneDev sc, SceneGradDev gr, ViewList vl, const ViewDev* __restrict__ views, CfgDev cfg,
+    const uint32_t* __restrict__ vis_mask, const float4* __restrict__ g2d) {
+  wait_prior_grid();
+  __shared__ ViewDev s_view;
+  __shared__ uint32_t s_any[kPbWords], s_first[kPbWords + 1];
+  __shared__ uint16_t s_list[kPbPrims];
+  const int64_t P = sc.P, p0 = (int64_t)blockIdx.x * kPbPrims;
+  const uint32_t w0 = (uint32_t)(p0 >> 5), n_words = (uint32_t)min((int64_t)kPbWords, (P + 31) / 32 - (int64_t)w0);
+  const ViewDev& vd = views[vl.idx[0]];
+  if (threadIdx.x < kPbWords) s_any[threadIdx.x] = threadIdx.x < n_words ? vis_mask[vd.mask_off + w0 + threadIdx.x] : 0u;
+  if (threadIdx.x == 0) s_view = vd;
+  __syncthreads();
+  if (threadIdx.x < 32) {  // the first list position of each word
+    const uint32_t n = threadIdx.x < kPbWords ? __popc(s_any[threadIdx.x]) : 0u;
+    uint32_t x = n;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, d);
+      if ((int)threadIdx.x >= d) x += y;
+    }
+    if (threadIdx.x < kPbWords) s_first[threadIdx.x] = x - n;
+    if (threadIdx.x == kPbWords - 1) s_first[kPbWords] = x;
+  }
+  __syncthreads();
+  const bool add = (cfg.flags & 4) != 0;  // add to the caller's running sum (UBS_FLAG_ACCUMULATE_GRADS)
+  const int nr = sc.rot_mode == 0 ? 4 : 3;
+  for (int i = threadIdx.x; i < kPbPrims; i += kPbThreads) {
+    const uint32_t any = s_any[i >> 5], bit = 1u << (i & 31);
+    if (any & bit) s_list[s_first[i >> 5] + __popc(any & (bit - 1u))] = (uint16_t)i;
+  }
+  __syncthreads();
+  const uint32_t n_items = s_first[kPbWords];
+  auto put = [&](float* dst, float v) { *dst = add ? *dst + v : v; };
+  for (uint32_t i = threadIdx.x; i < n_items; i += kPbThreads) {
+    const uint32_t l = s_list[i];
+    const int64_t p = p0 + l;
+    PrimIn<C> in;
+    load_prim_b<C>(sc, p, in);
+    PrimVI<C> vi;
+    prim_stage<C>(in, sc.rot_mode, vi);
+    PrimAcc<C> acc;
+    acc_zero<C>(acc);
+    const uint32_t r = s_view.rec_off + (uint32_t)p;
+    const float4 a = g2d[3 * (size_t)r], b = g2d[3 * (size_t)r + 1], c = g2d[3 * (size_t)r + 2];
+    const float g[10] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y};
+    prim_backward_view<C>(in, vi, s_view, cfg, g, acc);
+    PrimGrad<C> out;
+    prim_backward_final<C>(in, vi, sc.rot_mode, acc, out);
+    for (int j = 0; j < 3; ++j) put(gr.mean_x + j * P + p, out.mx[j]);
+    for (int j = 0; j < nr; ++j) put(gr.rot + j * P + p, out.rot[j]);
+    for (int j = 0; j < 3; ++j) put(gr.scale_x + j * P + p, out.s[j]);
+    for (int j = 0; j < 1 + C; ++j) put(gr.b + j * P + p, out.b[j]);
+    put(gr.opacity + p, out.o);
+    for (int j = 0; j < 3; ++j) put(gr.rgb + j * P + p, out.rgb[j]);
+    if constexpr (C > 0) {
+      for (int j = 0; j < C; ++j) put(gr.mean_q + j * P + p, out.mq[j]);
+      for (int j = 0; j < 3 * C; ++j) put(gr.L_qx + j * P + p, out.lqx[j]);
+      for (int j = 0; j < C * (C + 1) / 2; ++j) put(gr.L_q + j * P + p, out.lq[j]);
+    }
+  }
+  if (add) return;
+#pragma unroll 1
+  for (int i = threadIdx.x; i < kPbPrims; i += kPbThreads) {
+    const int64_t p = p0 + i;
+    if (p >= P || ((s_any[i >> 5] >> (i & 31)) & 1u)) continue;
+    for (int j = 0; j < 3; ++j) gr.mean_x[j * P + p] = 0.0f;
+    for (int j = 0; j < nr; ++j) gr.rot[j * P + p] = 0.0f;
+    for (int j = 0; j < 3; ++j) gr.scale_x[j * P + p] = 0.0f;
+    for (int j = 0; j < 1 + C; ++j) gr.b[j * P + p] = 0.0f;
+    gr.opacity[p] = 0.0f;
+    for (int j = 0; j < 3; ++j) gr.rgb[j * P + p] = 0.0f;
+    if constexpr (C > 0) {
+      for (int j = 0; j < C; ++j) gr.mean_q[j * P + p] = 0.0f;
+      for (int j = 0; j < 3 * C; ++j) gr.L_qx[j * P + p] = 0.0f;
+      for (int j = 0; j < C * (C + 1) / 2; ++j) gr.L_q[j * P + p] = 0.0f;
+    }
+  }
+}
 
 // Zeroes one scene's gradient planes (the primitives that no view sees keep
 // these zeros; the others are overwritten by prim_backward_kernel).
@@ -175,19 +268,24 @@ cudaError_t launch_prim_backward(const SceneDev& sc, const SceneGradDev& g, cons
   const uint32_t* tiles = (const uint32_t*)(ws + L.tiles);
   const float4* g2d = (const float4*)(ws + L.g2d);
   cudaError_t e = cudaSuccess;
-  if (vl.n <= 1) {  // one view: every primitive, directly
-    const unsigned blocks = (unsigned)nblk;
+  if (vl.n == 1 && sc.N > 3) {  // the drawn primitives of each CTA's range
+    const dim3 grid((unsigned)((sc.P + kPbPrims - 1) / kPbPrims));
+    const uint32_t* vis = (const uint32_t*)(ws + L.vis_mask);
     switch (sc.N) {
-      case 3: e = launch_dependent(prim_backward_kernel<0>, dim3(blocks), dim3(threads), smem, st, sc, g, vl, views, cfg, tiles, g2d); break;
-      case 4: e = launch_dependent(prim_backward_kernel<1>, dim3(blocks), dim3(threads), smem, st, sc, g, vl, views, cfg, tiles, g2d); break;
-      case 6: e = launch_dependent(prim_backward_kernel<3>, dim3(blocks), dim3(threads), smem, st, sc, g, vl, views, cfg, tiles, g2d); break;
-      case 7: e = launch_dependent(prim_backward_kernel<4>, dim3(blocks), dim3(threads), smem, st, sc, g, vl, views, cfg, tiles, g2d); break;
+      case 4: e = launch_dependent(prim_backward_drawn_kernel<1>, grid, dim3(kPbThreads), 0, st, sc, g, vl, views, cfg, vis, g2d); break;
+      case 6: e = launch_dependent(prim_backward_drawn_kernel<3>, grid, dim3(kPbThreads), 0, st, sc, g, vl, views, cfg, vis, g2d); break;
+      case 7: e = launch_dependent(prim_backward_drawn_kernel<4>, grid, dim3(kPbThreads), 0, st, sc, g, vl, views, cfg, vis, g2d); break;
       default: return cudaErrorInvalidValue;
     }
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
   }
-  // several views: the listed primitives, the others zeroed first unless accumulating
+  if (vl.n == 1) {  // N = 3: most primitives are drawn and an undrawn one costs little; every one, directly
+    e = launch_dependent(prim_backward_kernel<0>, dim3((unsigned)nblk), dim3(threads), smem, st, sc, g, vl, views,
+                         cfg, tiles, g2d);
+    return e != cudaSuccess ? e : cudaGetLastError();
+  }
+  // several views (or none: an empty list): the listed primitives, the others
+  // zeroed first unless accumulating
   if (!(cfg.flags & 4)) {
     e = launch_dependent(zero_scene_grads_kernel, dim3((unsigned)((sc.P + 255) / 256)), dim3(256), 0, st, g, sc.P,
                          sc.N - 3, sc.rot_mode == 0 ? 4 : 3);
