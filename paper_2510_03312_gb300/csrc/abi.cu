@@ -99,16 +99,18 @@ ubs_status make_layout(const ubs_problem* pr, Layout& L) {
     o = align256(o + bytes);
     return at;
   };
-  L.header = take(sizeof(Header));
   L.views = take(sizeof(ViewDev) * L.V);
   L.rec4 = take((size_t)L.R * kRecFloats * 4);
   L.key = take((size_t)L.R * 4);
   L.tiles = take((size_t)L.R * 4);
   L.rect = take((size_t)L.R * 8);
   L.g2d = take((size_t)L.R * kGradFloats * 4);
-  L.tcount = take((size_t)L.NT * kTileSub * 4 + 4 * 132 * 4 + kVisBlocks * 4);
+  L.tcount = take((size_t)L.NT * kTileSub * 4 + 4 * 132 * 4 + kVisBlocks * 4 + sizeof(Header));
   L.order_count = L.tcount + (size_t)L.NT * kTileSub * 4;
   L.vis_part = L.order_count + 4 * 132 * 4;
+  L.header = L.vis_part + kVisBlocks * 4;  // directly after: ubs_read_status copies both at once
+  static_assert(kTileSub * 4 % alignof(Header) == 0 && 4 * 132 * 4 % alignof(Header) == 0 &&
+                kVisBlocks * 4 % alignof(Header) == 0, "the header's alignment");
   L.cursor = take((size_t)L.NT * kTileSub * 4);
   L.vis_mask = take((size_t)L.mask_words * 4);
   L.bucket = take((size_t)L.cap * 4);
@@ -398,18 +400,20 @@ ubs_status ubs_read_status(const ubs_problem* pr, void* ws, size_t ws_bytes, ubs
   ubs_status st = prepare(pr, ws, ws_bytes, L);
   if (st != UBS_OK) return st;
   if (!out) return UBS_ERR_INVALID_ARG;
-  if (cudaStreamSynchronize(stream) != cudaSuccess) return UBS_ERR_CUDA;
-  Header h;
-  if (cudaMemcpy(&h, (char*)ws + L.header, sizeof(Header), cudaMemcpyDeviceToHost) != cudaSuccess)
+  struct {
+    uint32_t part[kVisBlocks];
+    Header h;
+  } s;
+  static_assert(offsetof(decltype(s), h) == kVisBlocks * 4, "as in the workspace");
+  if (cudaMemcpyAsync(&s, (char*)ws + L.vis_part, sizeof(s), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+      cudaStreamSynchronize(stream) != cudaSuccess)
     return UBS_ERR_CUDA;
+  const Header& h = s.h;
   out->status = (int32_t)h.status;
   out->reserved = 0;
-  uint32_t part[kVisBlocks];
-  if (cudaMemcpy(part, (char*)ws + L.vis_part, sizeof(part), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return UBS_ERR_CUDA;
   int64_t vis = 0;
   const uint32_t nb = L.R ? walk_blocks(L) : 0u;
-  for (uint32_t i = 0; i < nb; ++i) vis += part[i];
+  for (uint32_t i = 0; i < nb; ++i) vis += s.part[i];
   out->visible_records = vis;
   out->instances = (int64_t)h.n_inst;
   return UBS_OK;

@@ -64,7 +64,7 @@ struct SceneGradDev {
   float* rgb;
 };
 
-// Device status block at the start of the workspace.
+// Device status block (Layout::header).
 struct Header {
   uint32_t status;       // ubs_status of device-side work (0 = ok)
   uint32_t n_items;      // work items of the per-tile sort (0 after a capacity overflow)

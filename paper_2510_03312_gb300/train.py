@@ -10,7 +10,6 @@ diagonal of L_q = exp(raw), everything else the identity.
 """
 from __future__ import annotations
 
-import ctypes
 from dataclasses import dataclass
 
 import numpy as np
@@ -18,7 +17,7 @@ import torch
 
 from . import scenes as S
 from . import ubs as U
-from .raster import check_tensor, overlaps
+from .raster import check_tensor, current_stream, overlaps
 
 LAMBDA_SSIM = 0.2  # not stated in the paper; the value of 3DGS, whose loss this extends
 
@@ -102,7 +101,7 @@ class ImageLoss:
             raise ValueError("dL may not alias the image or the target")
         st = U.ubs_image_loss(self.widths, self.heights, image.data_ptr(), target.data_ptr(), self.lam,
                               dL.data_ptr(), self.loss.data_ptr(), self.ws_ptr, self.ws_bytes,
-                              ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+                              current_stream())
         if st != U.UBS_OK:
             raise U.UBSError(st, "ubs_image_loss")
         return self.loss
@@ -132,6 +131,9 @@ class Adam:
         for k, (lr, a, l1, row) in enumerate(self.table):
             self._planes[k].lr, self._planes[k].activation = lr, a
             self._planes[k].l1_weight, self._planes[k].noise_row = l1, row
+        self._planes_quiet = (U.ubs_adam_plane * K)(*self._planes)  # for steps without noise
+        for k in range(K):
+            self._planes_quiet[k].noise_row = -1
 
     def step(self, grad: torch.Tensor, noise: torch.Tensor | None = None):
         """One step with dL/d(activated params) ``grad``; ``noise`` [3, P] is the
@@ -144,15 +146,11 @@ class Adam:
         self.step_count += 1
         cfg = U.ubs_adam_config(self.tc.beta1, self.tc.beta2, self.tc.eps, self.step_count,
                                 self.tc.lambda_eps if noise is not None else 0.0)
-        planes = self._planes
-        if noise is None:
-            planes = (U.ubs_adam_plane * self.K)(*self._planes)
-            for k in range(self.K):
-                planes[k].noise_row = -1
+        planes = self._planes if noise is not None else self._planes_quiet
         st = U.ubs_adam_step(self.K, self.P, planes, cfg, self.raw.data_ptr(), self.act.data_ptr(),
                              grad.data_ptr(), self.m.data_ptr(), self.v.data_ptr(),
                              noise.data_ptr() if noise is not None else None,
-                             ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+                             current_stream())
         if st != U.UBS_OK:
             raise U.UBSError(st, "ubs_adam_step")
 
@@ -221,7 +219,7 @@ class Relocator:
         st = U.ubs_mcmc_relocate(o.K, o.P, self.opacity_row, self.threshold, o.act.data_ptr(), o.raw.data_ptr(),
                                  o.m.data_ptr(), o.v.data_ptr(), rand.data_ptr(), self.sources.data_ptr(),
                                  self.n_relocated.data_ptr(), self.ws_ptr, self.ws_bytes,
-                                 ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+                                 current_stream())
         if st != U.UBS_OK:
             raise U.UBSError(st, "ubs_mcmc_relocate")
         return self.sources, self.n_relocated
