@@ -112,6 +112,9 @@ ubs_status make_layout(const ubs_problem* pr, Layout& L) {
   static_assert(kTileSub * 4 % alignof(Header) == 0 && 4 * 132 * 4 % alignof(Header) == 0 &&
                 kVisBlocks * 4 % alignof(Header) == 0, "the header's alignment");
   L.cursor = take((size_t)L.NT * kTileSub * 4);
+  static_assert(kTileSub * 4 >= sizeof(uint4) + 4, "the tile descriptors take the cursors' place");
+  L.tile_desc = L.cursor;
+  L.tile_pix = L.cursor + (size_t)L.NT * sizeof(uint4);
   L.vis_mask = take((size_t)L.mask_words * 4);
   L.bucket = take((size_t)L.cap * 4);
   L.ivals = take((size_t)L.cap * 4);

@@ -89,7 +89,10 @@ struct Layout {
                      // the totals and cursors of the tile order and of the short lists' sort
                      // items [4 x 132], then the visible records per count block [kVisBlocks]
                      // (zeroed together by ubs_preprocess)
-  size_t cursor;     // next free slot of each (tile, sub-bucket) [kTileSub][NT]
+  size_t cursor;     // next free slot of each (tile, sub-bucket) [kTileSub][NT]; after the scatter, the
+                     // blend kernels' tile descriptors in its place (tile_desc, tile_pix)
+  size_t tile_desc;  // per tile (start, end, x0 | y0 << 16, W | H << 16): its list, first pixel and image size [NT]
+  size_t tile_pix;   // and the first pixel of its view [NT]
   size_t vis_mask;   // per view, a bit per primitive: visible (written whole by preprocess) [mask_words]
   size_t bucket;     // the instances grouped by tile, unordered within a tile [cap]
   size_t ivals;      // the sorted instance lists [cap]

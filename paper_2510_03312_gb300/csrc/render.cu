@@ -169,21 +169,15 @@ __device__ __forceinline__ void eval_pair2(float2 lx, float2 ly, const float4& A
   e.alpha = make_float2(fminf(amax, ex2_approx(ex.x)), fminf(amax, ex2_approx(ex.y)));
 }
 
-// The view holding global tile g: the last view whose first tile is at or
-// before g (views are numbered in tile order and view 0 starts at tile 0).
-// Called by a whole warp: a ballot over 32 views, after one over the first
-// views of 32-view chunks when there are more than 32 -- at most two
-// dependent loads, where a binary search takes log2(V).
-__device__ __forceinline__ int find_view_warp(const ViewDev* __restrict__ views, int V, uint32_t g) {
-  if (V == 1) return 0;
-  const int lane = threadIdx.x & 31;
-  int c = 0;
-  if (V > 32) {
-    const int i = lane * 32;
-    c = 31 - __clz(__ballot_sync(kFull, i < V && views[i].tile_off <= g));
-  }
-  const int i = c * 32 + lane;
-  return c * 32 + (31 - __clz(__ballot_sync(kFull, i < V && views[i].tile_off <= g)));
+// A tile as the binning's last kernel describes it: its list [start, end),
+// its first pixel, and its view's image.
+struct Tile {
+  uint32_t start, end;
+  int x0, y0, W, H;
+  size_t pix;  // first pixel of the view in the packed images
+};
+__device__ __forceinline__ Tile make_tile(const uint4& d, uint32_t pix) {
+  return Tile{d.x, d.y, (int)(d.z & 0xFFFFu), (int)(d.z >> 16), (int)(d.w & 0xFFFFu), (int)(d.w >> 16), pix};
 }
 
 // the warp's 8 x RB block (bx, by) within a TW-wide tile and this lane's
@@ -244,15 +238,13 @@ struct FwdSmem {
   Staged2 st[BS];
   float4 bb[BS];
   float rc[BS];
-  int v;
   uint32_t next;
 };
 
 struct FwdArgs {
-  const ViewDev* __restrict__ views;
-  int V;
   CfgDev cfg;
-  const uint32_t* __restrict__ tstart;
+  const uint4* __restrict__ desc;
+  const uint32_t* __restrict__ tpix;
   const uint32_t* __restrict__ ivals;
   const float4* __restrict__ rec4;
   float* __restrict__ image;
@@ -277,7 +269,7 @@ struct FwdArgs {
   uint32_t max_extra, max_slots;  // grid bounds: CTAs of extra segments and of slots, each looping
 };
 
-// One tile g, by the whole CTA (every thread calls it).  With SPLIT it
+// One tile, by the whole CTA (every thread calls it).  With SPLIT it
 // walks only the list positions [wbeg, wend) of the tile and, when `slot`
 // is given, writes each pixel's state there (colour, T, last contributor
 // and whether the pixel terminated) instead of the image: the part of one
@@ -287,31 +279,23 @@ struct FwdArgs {
 // every pixel of the tile stops: no pixel's result can use it.  A segment
 // whose walk ends every pixel records its index there.
 template <int TW, int TH, bool COUNT, bool SPLIT = false>
-__device__ __forceinline__ void fwd_tile(const FwdArgs& A, uint32_t g, FwdSmem<TW, TH>& sm, uint32_t wbeg = 0,
+__device__ __forceinline__ void fwd_tile(const FwdArgs& A, const Tile& v, FwdSmem<TW, TH>& sm, uint32_t wbeg = 0,
                                          uint32_t wend = 0xffffffffu, float4* slot = nullptr,
                                          uint32_t* slot_l = nullptr, const uint32_t* resume = nullptr,
                                          uint32_t* term = nullptr, uint32_t seg = 0) {
   constexpr int NT = FwdSmem<TW, TH>::NT, BS = FwdSmem<TW, TH>::BS;
   const CfgDev& cfg = A.cfg;
-  uint32_t start = A.tstart[g], end = A.tstart[g + 1];  // loaded while warp 0 finds the view
+  uint32_t start = v.start, end = v.end;
   const uint32_t list0 = start;  // positions are numbered from the tile list's first entry
   if constexpr (SPLIT) {
     start = min(end, list0 + wbeg);
     end = min(end, list0 + min(wend, 0xffffffffu - list0));
   }
-  if (threadIdx.x < 32) {
-    const int vi = find_view_warp(A.views, A.V, g);
-    if (threadIdx.x == 0) sm.v = vi;
-  }
-  __syncthreads();
-  const ViewDev& v = A.views[sm.v];
-  const uint32_t lt = g - v.tile_off;
-  const int tx = lt % v.tiles_x, ty = lt / v.tiles_x;
   int lx, ly, bx, by;
   pixel_of<TW, 8>(lx, ly, bx, by);
-  const int x = tx * TW + lx, y0 = ty * TH + ly, y1 = y0 + 4;
+  const int x = v.x0 + lx, y0 = v.y0 + ly, y1 = y0 + 4;
   const bool in0 = x < v.W && y0 < v.H, in1 = x < v.W && y1 < v.H;
-  const float ox = (float)(tx * TW), oy = (float)(ty * TH);
+  const float ox = (float)v.x0, oy = (float)v.y0;
   const float2 fx = make_float2((float)lx + 0.5f, (float)lx + 0.5f);  // pixel centres, tile-relative
   const float2 fy = make_float2((float)ly + 0.5f, (float)(ly + 4) + 0.5f);
   const float wx0 = (float)bx + 0.5f, wx1 = wx0 + 7.0f, wy0 = (float)by + 0.5f, wy1 = wy0 + 7.0f;
@@ -428,17 +412,17 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& A, uint32_t g, FwdSmem<T
     }
   }
   const size_t plane = (size_t)v.W * v.H;
-  float* img = A.image + (size_t)v.pix_off * 3;
+  float* img = A.image + v.pix * 3;
   if (in0) {
     const size_t pix = (size_t)y0 * v.W + x;
     img[pix] = fmaf(T.x, cfg.bg[0], C0.x);
     img[plane + pix] = fmaf(T.x, cfg.bg[1], C1.x);
     img[2 * plane + pix] = fmaf(T.x, cfg.bg[2], C2.x);
-    A.Tfin[v.pix_off + pix] = T.x;
-    A.lastc[v.pix_off + pix] = last0;
+    A.Tfin[v.pix + pix] = T.x;
+    A.lastc[v.pix + pix] = last0;
     if constexpr (COUNT) {
-      A.pairs[v.pix_off + pix] = np0;
-      A.visited[v.pix_off + pix] = nv;
+      A.pairs[v.pix + pix] = np0;
+      A.visited[v.pix + pix] = nv;
     }
   }
   if (in1) {
@@ -446,13 +430,24 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs& A, uint32_t g, FwdSmem<T
     img[pix] = fmaf(T.y, cfg.bg[0], C0.y);
     img[plane + pix] = fmaf(T.y, cfg.bg[1], C1.y);
     img[2 * plane + pix] = fmaf(T.y, cfg.bg[2], C2.y);
-    A.Tfin[v.pix_off + pix] = T.y;
-    A.lastc[v.pix_off + pix] = last1;
+    A.Tfin[v.pix + pix] = T.y;
+    A.lastc[v.pix + pix] = last1;
     if constexpr (COUNT) {
-      A.pairs[v.pix_off + pix] = np1;
-      A.visited[v.pix_off + pix] = nv;
+      A.pairs[v.pix + pix] = np1;
+      A.visited[v.pix + pix] = nv;
     }
   }
+}
+
+// The t-th tile of a blend grid, in the order bin_sort made where the lists
+// are dense; d and pix hold tile t's descriptor and get the returned tile's.
+template <class Args>
+__device__ __forceinline__ uint32_t tile_at(const Args& A, uint32_t t, uint4& d, uint32_t& pix) {
+  if (!(A.tile_order && order_dense(A.hdr, A.n_tiles, A.cap))) return t;
+  const uint32_t g = A.tile_order[t];
+  d = A.desc[g];
+  pix = A.tpix[g];
+  return g;
 }
 
 // The grid form: one CTA per tile, in bin_sort's tile order where the lists
@@ -465,8 +460,12 @@ __global__ void __launch_bounds__(TW * TH / 2, (TW * TH / 2 >= 128 ? 1024 / (TW 
     render_fwd_kernel(FwdArgs A) {
   wait_prior_grid();
   __shared__ FwdSmem<TW, TH> sm;
-  if (A.hdr->status != 0) return;
   uint32_t t = blockIdx.x;
+  // the tile's descriptor, with the header's words and not after them
+  const uint32_t t0 = SPLIT && t >= A.n_tiles ? 0u : t;
+  uint4 d = A.desc[t0];
+  uint32_t pix = A.tpix[t0];
+  if (A.hdr->status != 0) return;
   if constexpr (SPLIT) {
     constexpr int TP = TW * TH;  // pixels per tile: the float4 pairs of a slot
     if (t >= A.n_tiles) {
@@ -479,24 +478,25 @@ __global__ void __launch_bounds__(TW * TH / 2, (TW * TH / 2 >= 128 ? 1024 / (TW 
         const uint4 sp = A.split_list[i];
         const uint32_t k = e - sp.w + 1;
         const size_t at = (size_t)(sp.y + k) * TP;
-        fwd_tile<TW, TH, COUNT, true>(A, sp.x, sm, k * len, (k + 1) * len, A.seg_c + at, A.seg_l + at, nullptr,
+        fwd_tile<TW, TH, COUNT, true>(A, make_tile(A.desc[sp.x], A.tpix[sp.x]), sm, k * len, (k + 1) * len, A.seg_c + at, A.seg_l + at, nullptr,
                                       A.split_term + i, k);
         __syncthreads();  // shared memory is free for the next segment
       }
       return;
     }
-    const uint32_t g = A.tile_order && order_dense(A.hdr, A.n_tiles, A.cap) ? A.tile_order[t] : t;
+    const uint32_t g = tile_at(A, t, d, pix);
     const uint32_t i = A.tile_split[g];
+    const Tile v = make_tile(d, pix);
     if (i != 0xffffffffu) {
       const size_t at = (size_t)A.split_list[i].y * TP;
-      fwd_tile<TW, TH, COUNT, true>(A, g, sm, 0, A.hdr->ctr[kCtrSegLen], A.seg_c + at, A.seg_l + at, nullptr,
+      fwd_tile<TW, TH, COUNT, true>(A, v, sm, 0, A.hdr->ctr[kCtrSegLen], A.seg_c + at, A.seg_l + at, nullptr,
                                     A.split_term + i, 0);
     }
     else
-      fwd_tile<TW, TH, COUNT, true>(A, g, sm);
+      fwd_tile<TW, TH, COUNT, true>(A, v, sm);
   } else {
-    const uint32_t g = A.tile_order && order_dense(A.hdr, A.n_tiles, A.cap) ? A.tile_order[t] : t;
-    fwd_tile<TW, TH, COUNT>(A, g, sm);
+    tile_at(A, t, d, pix);
+    fwd_tile<TW, TH, COUNT>(A, make_tile(d, pix), sm);
   }
 }
 
@@ -569,8 +569,10 @@ __global__ void __launch_bounds__(TW * TH / 2, (TW * TH / 2 >= 128 ? 1024 / (TW 
     if (threadIdx.x == 0) sm.next = atomicAdd(A.queue, 1u);
     __syncthreads();  // also: every thread is done with the previous tile's shared memory
     const uint32_t t = sm.next;
+    __syncthreads();  // read by all before the next one is written: an empty tile has no barrier
     if (t >= A.n_tiles) break;
-    fwd_tile<TW, TH, COUNT>(A, dense ? A.tile_order[t] : t, sm);
+    const uint32_t g = dense ? A.tile_order[t] : t;
+    fwd_tile<TW, TH, COUNT>(A, make_tile(A.desc[g], A.tpix[g]), sm);
   }
   if (threadIdx.x == 0 && atomicAdd(A.queue + 1, 1u) == gridDim.x - 1) {
     A.queue[0] = 0;  // every CTA has taken its last tile
@@ -703,7 +705,7 @@ __global__ void __launch_bounds__(TW * TH / 2, (TW * TH / 2 >= 128 ? 1024 / (TW 
     const bool any = end[threadIdx.x] == (k | kSegEnded) || end[threadIdx.x + TP / 2] == (k | kSegEnded);
     if (__syncthreads_or(any) == 0) continue;  // no pixel ends here; also: shared memory is free for this segment
     const size_t at = (size_t)s * TP;
-    fwd_tile<TW, TH, false, true>(A, sp.x, sm, k * len, (k + 1) * len, A.seg_c + at, A.seg_l + at, end, nullptr, k);
+    fwd_tile<TW, TH, false, true>(A, make_tile(A.desc[sp.x], A.tpix[sp.x]), sm, k * len, (k + 1) * len, A.seg_c + at, A.seg_l + at, end, nullptr, k);
   }
 }
 
@@ -717,7 +719,6 @@ template <int TW, int TH>
 __global__ void __launch_bounds__(32 * kJoinW) split_finish_kernel(FwdArgs A) {
   wait_prior_grid();
   constexpr int TP = TW * TH, CPT = TP / 32;
-  __shared__ int s_v;
   __shared__ float4 s_c[kJoinW][32];
   if (A.hdr->status != 0) return;
   const CfgDev& cfg = A.cfg;
@@ -725,11 +726,7 @@ __global__ void __launch_bounds__(32 * kJoinW) split_finish_kernel(FwdArgs A) {
   const uint32_t n_items = A.hdr->ctr[4] * CPT;
   for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
     const uint4 sp = A.split_list[it / CPT];
-    const uint32_t g = sp.x, px = (it % CPT) * 32 + lane;
-    if (w == 0) {
-      const int vi = find_view_warp(A.views, A.V, g);
-      if (lane == 0) s_v = vi;
-    }
+    const uint32_t px = (it % CPT) * 32 + lane;
     float4* my = A.seg_c + (size_t)sp.y * TP + px;
     const uint32_t* my_l = A.seg_l + (size_t)sp.y * TP + px;
     const uint32_t end = A.seg_end[(size_t)(it / CPT) * TP + px];
@@ -749,10 +746,8 @@ __global__ void __launch_bounds__(32 * kJoinW) split_finish_kernel(FwdArgs A) {
     s_c[w][lane] = make_float4(C0, C1, C2, 0.0f);
     __syncthreads();
     if (w == 0) {
-      const ViewDev& v = A.views[s_v];
-      const uint32_t lt = g - v.tile_off;
-      const int tx = lt % v.tiles_x, ty = lt / v.tiles_x;
-      const int x = tx * TW + (int)(px % TW), y = ty * TH + (int)(px / TW);
+      const Tile v = make_tile(A.desc[sp.x], A.tpix[sp.x]);
+      const int x = v.x0 + (int)(px % TW), y = v.y0 + (int)(px / TW);
       if (x < v.W && y < v.H) {
         for (int h = 1; h < kJoinW; ++h) {
           C0 += s_c[h][lane].x;
@@ -760,12 +755,12 @@ __global__ void __launch_bounds__(32 * kJoinW) split_finish_kernel(FwdArgs A) {
           C2 += s_c[h][lane].z;
         }
         const size_t plane = (size_t)v.W * v.H, pix = (size_t)y * v.W + x;
-        float* img = A.image + (size_t)v.pix_off * 3;
+        float* img = A.image + v.pix * 3;
         img[pix] = fmaf(T, cfg.bg[0], C0);
         img[plane + pix] = fmaf(T, cfg.bg[1], C1);
         img[2 * plane + pix] = fmaf(T, cfg.bg[2], C2);
-        A.Tfin[v.pix_off + pix] = T;
-        A.lastc[v.pix_off + pix] = my_l[(end & kSegEnded) ? (size_t)kend * TP : 0];
+        A.Tfin[v.pix + pix] = T;
+        A.lastc[v.pix + pix] = my_l[(end & kSegEnded) ? (size_t)kend * TP : 0];
       }
     }
     float b0 = T * cfg.bg[0], b1 = T * cfg.bg[1], b2 = T * cfg.bg[2];
@@ -855,10 +850,9 @@ struct BwdSmem {
 };
 
 struct BwdArgs {
-  const ViewDev* __restrict__ views;
-  int V;
   CfgDev cfg;
-  const uint32_t* __restrict__ tstart;
+  const uint4* __restrict__ desc;
+  const uint32_t* __restrict__ tpix;
   const uint32_t* __restrict__ ivals;
   const float4* __restrict__ rec4;
   const float* __restrict__ dLdimg;
@@ -878,26 +872,22 @@ struct BwdArgs {
   uint32_t max_extra;  // CTAs of extra segments (per 8x8 block), each looping
 };
 
-// One 8x8 block wb of tile g, by one warp.  With SPLIT and a slot, only the
+// One 8x8 block wb of a tile, by one warp.  With SPLIT and a slot, only the
 // list positions [wbeg, wend) of one segment are walked, from the
 // transmittance and colour behind at the segment's end that the forward's
 // merge left in the slot.
 template <int TW, int TH, bool SPLIT = false>
-__device__ __forceinline__ void bwd_block(const BwdArgs& A, uint32_t g, int wb, BwdSmem& sm, uint32_t wbeg = 0,
+__device__ __forceinline__ void bwd_block(const BwdArgs& A, const Tile& v, int wb, BwdSmem& sm, uint32_t wbeg = 0,
                                           uint32_t wend = 0xffffffffu, const float4* slot = nullptr) {
   constexpr int WB = BwdSmem::WB;
   constexpr int WPR = TW / 8;  // blocks per row of the tile
   const CfgDev& cfg = A.cfg;
   const int lane = threadIdx.x & 31;
-  const uint32_t start = A.tstart[g], end = A.tstart[g + 1];  // loaded while the view is found
-  const int vi = find_view_warp(A.views, A.V, g);
+  const uint32_t start = v.start, end = v.end;
   if (start == end) return;  // an empty list: no pixel of the tile has a contributor
-  const ViewDev& v = A.views[vi];
-  const uint32_t lt = g - v.tile_off;
-  const int tx = lt % v.tiles_x, ty = lt / v.tiles_x;
   const int bx = (wb % WPR) * 8, by = (wb / WPR) * 8;
   const int lx = bx + (lane & 7), ly = by + (lane >> 3);
-  const int x = tx * TW + lx;
+  const int x = v.x0 + lx;
   // per-pixel state of the lane's two pixels, packed: .x row ly, .y row ly + 4
   const float2 fx = make_float2((float)lx + 0.5f, (float)lx + 0.5f);
   const float2 fy = make_float2((float)ly + 0.5f, (float)(ly + 4) + 0.5f);
@@ -908,23 +898,23 @@ __device__ __forceinline__ void bwd_block(const BwdArgs& A, uint32_t g, int wb, 
   uint32_t last0 = 0, last1 = 0;
   {
     const size_t plane = (size_t)v.W * v.H;
-    const float* gi = A.dLdimg + (size_t)v.pix_off * 3;
-    const int y0 = ty * TH + ly, y1 = y0 + 4;
+    const float* gi = A.dLdimg + v.pix * 3;
+    const int y0 = v.y0 + ly, y1 = y0 + 4;
     if (x < v.W && y0 < v.H) {
       const size_t pix = (size_t)y0 * v.W + x;
       G0.x = gi[pix];
       G1.x = gi[plane + pix];
       G2.x = gi[2 * plane + pix];
-      T.x = A.Tfin[v.pix_off + pix];
-      last0 = A.lastc[v.pix_off + pix];
+      T.x = A.Tfin[v.pix + pix];
+      last0 = A.lastc[v.pix + pix];
     }
     if (x < v.W && y1 < v.H) {
       const size_t pix = (size_t)y1 * v.W + x;
       G0.y = gi[pix];
       G1.y = gi[plane + pix];
       G2.y = gi[2 * plane + pix];
-      T.y = A.Tfin[v.pix_off + pix];
-      last1 = A.lastc[v.pix_off + pix];
+      T.y = A.Tfin[v.pix + pix];
+      last1 = A.lastc[v.pix + pix];
     }
   }
   if constexpr (SPLIT) {
@@ -945,32 +935,38 @@ __device__ __forceinline__ void bwd_block(const BwdArgs& A, uint32_t g, int wb, 
       B2.y = s1.z;
     }
   }
+  const float ox = (float)v.x0, oy = (float)v.y0;
+  const float wx0 = (float)bx + 0.5f, wx1 = wx0 + 7.0f, wy0 = (float)by + 0.5f, wy1 = wy0 + 7.0f;
+  const float lg2_amin = lg2_approx(cfg.amin);
+  // stages list position i in this lane's entry; whether its support meets the block
+  auto stage = [&](uint32_t i) {
+    const uint32_t r = record_id(A.ivals[start + i], A.R, cfg, A.hdr);
+    Staged st;
+    float4 box;
+    float rc;
+    stage_record(A.rec4, r, ox, oy, lg2_amin, st, box, rc);
+    sm.rec[lane] = r;
+    sm.st[lane] = pack_staged(st);
+    return box_hits(box, wx0, wx1, wy0, wy1) && ellipse_hits(st.p, st.q.x, rc, wx0, wx1, wy0, wy1);
+  };
+  // a list of one batch is staged whole while the pixels' values arrive: its
+  // last contributor only cuts it short
+  const bool whole = !SPLIT && end - start <= (uint32_t)WB;
+  bool whole_hit = false;
+  if (whole && lane < (int)(end - start)) whole_hit = stage(lane);
   uint32_t wlast = __reduce_max_sync(kFull, max(last0, last1));
   if constexpr (SPLIT) {
     wlast = min(wlast, wend);
     if (wlast <= wbeg) return;
   }
   if (wlast == 0) return;
-  const float ox = (float)(tx * TW), oy = (float)(ty * TH);
-  const float wx0 = (float)bx + 0.5f, wx1 = wx0 + 7.0f, wy0 = (float)by + 0.5f, wy1 = wy0 + 7.0f;
-  const float lg2_amin = lg2_approx(cfg.amin);
   const float2 one = make_float2(1.0f, 1.0f), neg1 = make_float2(-1.0f, -1.0f);
   const int wslot = writer_of(lane);
   const int wfirst = SPLIT ? (int)wbeg : 0;
   for (int hi = (int)wlast; hi > wfirst; hi -= WB) {
     const int lo = hi - WB > wfirst ? hi - WB : wfirst;
     const int n = hi - lo;
-    bool listed = false;
-    if (lane < n) {
-      const uint32_t r = record_id(A.ivals[start + lo + lane], A.R, cfg, A.hdr);
-      Staged st;
-      float4 box;
-      float rc;
-      stage_record(A.rec4, r, ox, oy, lg2_amin, st, box, rc);
-      sm.rec[lane] = r;
-      sm.st[lane] = pack_staged(st);
-      listed = box_hits(box, wx0, wx1, wy0, wy1) && ellipse_hits(st.p, st.q.x, rc, wx0, wx1, wy0, wy1);
-    }
+    const bool listed = lane < n && (whole ? whole_hit : stage((uint32_t)(lo + lane)));
     const unsigned lm = __ballot_sync(kFull, listed);
     __syncwarp();
     unsigned touched = 0;  // entries the block used (warp-uniform)
@@ -1059,9 +1055,13 @@ __global__ void __launch_bounds__(32, 32)  // 64 registers: 32 one-warp CTAs per
   wait_prior_grid();
   constexpr int BPT = TW * TH / 64;  // 8x8 blocks per tile
   __shared__ BwdSmem sm;
-  if (A.hdr->status != 0) return;
   uint32_t t = blockIdx.x / BPT;
   const int wb = blockIdx.x % BPT;
+  // the tile's descriptor, with the header's words and not after them
+  const uint32_t t0 = SPLIT ? (t < A.max_extra ? 0u : t - A.max_extra) : t;
+  uint4 d = A.desc[t0];
+  uint32_t pix = A.tpix[t0];
+  if (A.hdr->status != 0) return;
   if constexpr (SPLIT) {
     constexpr int TP = TW * TH;
     if (t < A.max_extra) {
@@ -1069,22 +1069,22 @@ __global__ void __launch_bounds__(32, 32)  // 64 registers: 32 one-warp CTAs per
       for (uint32_t e = t; e < n_extra; e += A.max_extra) {
         const uint4 sp = A.split_list[A.ext_owner[e]];
         const uint32_t k = e - sp.w + 1;
-        bwd_block<TW, TH, true>(A, sp.x, wb, sm, k * len, (k + 1) * len,
+        bwd_block<TW, TH, true>(A, make_tile(A.desc[sp.x], A.tpix[sp.x]), wb, sm, k * len, (k + 1) * len,
                                 A.seg_c + (size_t)(sp.y + k) * TP);
         __syncwarp();
       }
       return;
     }
-    t -= A.max_extra;
-    const uint32_t g = A.tile_order && order_dense(A.hdr, A.n_tiles, A.cap) ? A.tile_order[t] : t;
+    const uint32_t g = tile_at(A, t0, d, pix);
     const uint32_t i = A.tile_split[g];
+    const Tile v = make_tile(d, pix);
     if (i != 0xffffffffu)
-      bwd_block<TW, TH, true>(A, g, wb, sm, 0, A.hdr->ctr[kCtrSegLen], A.seg_c + (size_t)A.split_list[i].y * TP);
+      bwd_block<TW, TH, true>(A, v, wb, sm, 0, A.hdr->ctr[kCtrSegLen], A.seg_c + (size_t)A.split_list[i].y * TP);
     else
-      bwd_block<TW, TH, true>(A, g, wb, sm);
+      bwd_block<TW, TH, true>(A, v, wb, sm);
   } else {
-    const uint32_t g = A.tile_order && order_dense(A.hdr, A.n_tiles, A.cap) ? A.tile_order[t] : t;
-    bwd_block<TW, TH>(A, g, wb, sm);
+    tile_at(A, t0, d, pix);
+    bwd_block<TW, TH>(A, make_tile(d, pix), wb, sm);
   }
 }
 
@@ -1108,8 +1108,9 @@ __global__ void __launch_bounds__(32, 32)
     t = __shfl_sync(kFull, t, 0);
     if (t >= A.n_tiles) break;
     const uint32_t g = dense ? A.tile_order[t] : t;
+    const Tile v = make_tile(A.desc[g], A.tpix[g]);
     for (int wb = 0; wb < BPT; ++wb) {
-      bwd_block<TW, TH>(A, g, wb, sm);
+      bwd_block<TW, TH>(A, v, wb, sm);
       __syncwarp();
     }
   }
@@ -1196,10 +1197,9 @@ cudaError_t fwd_split(const FwdArgs& args, const Layout& L, char* ws, cudaStream
 template <int TW, int TH>
 cudaError_t fwd_t(const Layout& L, const CfgDev& cfg, char* ws, float* image, cudaStream_t st) {
   FwdArgs a;
-  a.views = (const ViewDev*)(ws + L.views);
-  a.V = L.V;
   a.cfg = cfg;
-  a.tstart = (const uint32_t*)(ws + L.tstart);
+  a.desc = (const uint4*)(ws + L.tile_desc);
+  a.tpix = (const uint32_t*)(ws + L.tile_pix);
   a.ivals = sorted_instances(L, ws);
   a.rec4 = (const float4*)(ws + L.rec4);
   a.image = image;
@@ -1233,10 +1233,9 @@ cudaError_t fwd_t(const Layout& L, const CfgDev& cfg, char* ws, float* image, cu
 template <int TW, int TH>
 cudaError_t bwd_t(const Layout& L, const CfgDev& cfg, char* ws, const float* dL, cudaStream_t st) {
   BwdArgs a;
-  a.views = (const ViewDev*)(ws + L.views);
-  a.V = L.V;
   a.cfg = cfg;
-  a.tstart = (const uint32_t*)(ws + L.tstart);
+  a.desc = (const uint4*)(ws + L.tile_desc);
+  a.tpix = (const uint32_t*)(ws + L.tile_pix);
   a.ivals = sorted_instances(L, ws);
   a.rec4 = (const float4*)(ws + L.rec4);
   a.dLdimg = dL;
