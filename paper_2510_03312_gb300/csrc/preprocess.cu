@@ -95,81 +95,171 @@ __global__ void __launch_bounds__(256) preprocess_kernel(SceneDev sc, ViewList v
   }
 }
 
-// Scenes with query dimensions (N > 3): the conditioning runs per (view,
-// primitive) as in preprocess_kernel, but only the records that pass the
-// early tests (view_candidate) are projected, from a per-warp queue in
-// shared memory, 32 at a time.  Where the query culls most records (o(q)
-// below alpha_min), the projection -- over half of a record's arithmetic --
-// then runs on full warps instead of on the few lanes whose record survives.
-// The projection of a queued record is the same arithmetic on the same
-// values as in view_stage.
-constexpr int kQCap = 64;   // queue entries per warp: 31 carried over + 32 new
-constexpr int kQWarps = 8;  // warps per CTA (256 threads)
-// Held to 80 registers (three CTAs per SM, from two at 108-116): the
-// kernel's dependent float32 chains need the warps (the 16-view N=6 batch
-// 253 -> 232 us, the 8-view N=7 one 99 -> 91 us).
+// Scenes with query dimensions (N > 3).  The query culls most records (o(q)
+// below alpha_min: 6% of a 16-view N=6 batch is drawn, 2% of an N=7 one), and
+// the exact conditioning costs some 300 instructions a record, most of them
+// the correctly rounded divisions, square root, exp and log whose float32
+// results the decisions follow.  So every (view, primitive) is first put to a
+// cheap test, certain_cull, that no record the rule set draws can fail; the
+// records that pass go into a per-warp queue in shared memory, and whenever 32
+// are queued each lane takes one through the rule set's own conditioning,
+// tests and projection, from the owner's values in shared memory.  A lane's
+// arithmetic on a queued record is that of view_stage, so the outputs are the
+// same bits.
+// Bound by instruction issue; 16 views of 500K N=6 primitives 195 us with the
+// conditioning of every record on its own lane, 152 us so; 8 views of 300K
+// N=7 71 -> 53.  What is left is the view-independent stage and the queued
+// records.
+constexpr int kQThreads = 128, kQWarps = kQThreads / 32;
+constexpr int kQCap = 64;  // queue entries per warp: 31 carried over + 32 new
+
+// What certain_cull needs of a primitive.
+template <int C>
+struct CullPrim {
+  float mx[3], mq[C];
+  float rl[C];                 // 1 / L^_kk
+  float lo[C * (C - 1) / 2 + 1];  // L^_km, m < k
+  float b8[C];                 // 8 beta_qk
+  float below;                 // the exponent below which o(q) is certain to fall below alpha_min
+};
+
+// Whether the record's exponent bound E_ub (see view_condition) is certain to
+// lie below cull_below, from approximate y: y_k = (delta_k - sum L^_km y_m) /
+// L^_kk with err_k a bound on its distance from the rule set's float32 y_k:
+// the view direction's approximate normalisation and the roundings of both
+// are within 2e-6 (1 + |delta_k|) and 2e-6 of each term (a dozen times the
+// 1e-7 each operation can add), carried through the substitution.  The bound
+// is taken at |y_k| - err_k, its negative and positive parts scaled by
+// 1 -+ 1e-5, and `below` is 0.01 under cull_below, for the roundings of the
+// sums.  Comparisons with NaN (a
+// primitive at the camera, overflows) are false: such records are queued.
+template <int C>
+__device__ __forceinline__ bool certain_cull(const CullPrim<C>& p, const float (&cam)[3], float time) {
+  float q[C];
+  int qi = 0;
+  if constexpr (C == 1 || C == 4) q[qi++] = time;
+  if constexpr (C >= 3) {
+    const float v0 = p.mx[0] - cam[0], v1 = p.mx[1] - cam[1], v2 = p.mx[2] - cam[2];
+    float rn;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rn) : "f"(fmaf(v0, v0, fmaf(v1, v1, v2 * v2))));
+    q[qi++] = v0 * rn;
+    q[qi++] = v1 * rn;
+    q[qi++] = v2 * rn;
+  }
+  float y[C], err[C], E = 0.0f;
+#pragma unroll
+  for (int k = 0; k < C; ++k) {
+    const float d = q[k] - p.mq[k];
+    float a = d, e = fmaf(2e-6f, fabsf(d), 2e-6f);
+#pragma unroll
+    for (int m = 0; m < k; ++m) {
+      const float l = p.lo[k * (k - 1) / 2 + m];
+      a = fmaf(-l, y[m], a);
+      e = fmaf(fabsf(l), fmaf(2e-6f, fabsf(y[m]), err[m]), e);
+    }
+    y[k] = a * p.rl[k];
+    err[k] = fmaf(2e-6f, fabsf(y[k]), e * p.rl[k]);
+    const float ylo = fmaxf(fabsf(y[k]) - err[k], 0.0f);
+    // 4 beta (ln 2 - 2 y^2), in units of 8 beta
+    E = fmaf(p.b8[k], fmaf(-(1.0f - 1e-5f) * ylo, ylo, 0.5f * 0.69314718f * (1.0f + 1e-5f)), E);
+  }
+  return E < p.below;
+}
+
+// The queued record's primitive: the fields of PrimIn and PrimVI that the
+// conditioning and the projection read, a float per lane each.
+template <int C>
+struct QFields {
+  static constexpr int kMx = 0, kMq = 3, kLh = kMq + C, kW3 = kLh + C * (C + 1) / 2, kBq = kW3 + 3 * C, kO = kBq + C,
+                       kSc = kO + 1, kBx = kSc + 6, kRgb = kBx + 1, kBelow = kRgb + 3, kN = kBelow + 1;
+};
 
 template <int C>
-__global__ void __launch_bounds__(256, 3) preprocess_queued_kernel(SceneDev sc, ViewList vl,
-                                                                const ViewDev* __restrict__ views, CfgDev cfg,
-                                                                float4* __restrict__ rec4, uint32_t* __restrict__ key,
-                                                                uint32_t* __restrict__ tiles, uint2* __restrict__ rect,
-                                                                uint32_t* __restrict__ vis_mask,
-                                                                uint32_t* __restrict__ act_list, uint32_t* act_count,
-                                                                uint32_t* __restrict__ zero, uint32_t nzero) {
+__global__ void __launch_bounds__(kQThreads, 6) preprocess_queued_kernel(
+    SceneDev sc, ViewList vl, const ViewDev* __restrict__ views, CfgDev cfg, float4* __restrict__ rec4,
+    uint32_t* __restrict__ key, uint32_t* __restrict__ tiles, uint2* __restrict__ rect,
+    uint32_t* __restrict__ vis_mask, uint32_t* __restrict__ act_list, uint32_t* act_count,
+    uint32_t* __restrict__ zero, uint32_t nzero) {
   wait_prior_grid();
   zero_words(zero, nzero);
+  using F = QFields<C>;
   extern __shared__ ViewDev s_views[];
-  // per warp: the lanes' view-independent values (mean, Sigma, beta_x, rgb),
-  // and the queue (record, view | owner lane << 16, shift, o(q))
-  __shared__ float s_prim[kQWarps][13][32];
-  __shared__ float s_qf[kQWarps][4][kQCap];
-  __shared__ uint32_t s_qr[kQWarps][kQCap], s_qk[kQWarps][kQCap];
+  __shared__ float s_prim[kQWarps][F::kN][32];
+  __shared__ uint32_t s_q[kQWarps][kQCap];         // view | owner lane << 16
   __shared__ uint32_t s_any[kQWarps];
-  __shared__ uint32_t s_vis[kQWarps][kMaxViews];  // per warp and view: the visibility mask word
-  for (int i = threadIdx.x; i < vl.n; i += blockDim.x) s_views[i] = views[vl.idx[i]];
+  __shared__ uint32_t s_vis[kQWarps][kMaxViews];   // per warp and view: the visibility mask word
+  for (int i = threadIdx.x; i < vl.n; i += kQThreads) s_views[i] = views[vl.idx[i]];
   if (threadIdx.x < kQWarps) s_any[threadIdx.x] = 0;
-  for (int i = threadIdx.x; i < kQWarps * vl.n; i += blockDim.x) s_vis[i / vl.n][i % vl.n] = 0;
+  for (int i = threadIdx.x; i < kQWarps * vl.n; i += kQThreads) s_vis[i / vl.n][i % vl.n] = 0;
   __syncthreads();
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t p = (int64_t)blockIdx.x * kQThreads + threadIdx.x;
   const bool live = p < sc.P;  // every lane stays: the queue is warp-synchronous
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t p0 = (uint32_t)(p - lane);  // the warp's first primitive (P is below 2^31)
   const unsigned lt = (1u << lane) - 1u;
   float(*prim)[32] = s_prim[w];
-  float(*qf)[kQCap] = s_qf[w];
-  uint32_t* qr = s_qr[w];
-  uint32_t* qk = s_qk[w];
-  PrimIn<C> in;
-  PrimVI<C> vi;
-  // the log-opacity bound below which a record is certainly culled (see
-  // view_condition): approximate log and quotient, inside the bound's margin
-  float cull_below = -INFINITY;
+  uint32_t* queue = s_q[w];
+  CullPrim<C> cp;
+  cp.below = -INFINITY;  // no certain cull
   if (live) {
+    PrimIn<C> in;
+    PrimVI<C> vi;
     load_prim<C>(sc, p, in);
     prim_stage<C>(in, sc.rot_mode, vi);
+    // the log-opacity bound below which a record is certainly culled (see
+    // view_condition): approximate log and quotient, inside the bound's margin
+    float cull_below = -INFINITY;
     if (cfg.amin > 0.0f) cull_below = __logf(__fdividef(cfg.amin, in.o)) - 0.01f;
-    for (int i = 0; i < 3; ++i) prim[i][lane] = in.mx[i];
-    for (int i = 0; i < 6; ++i) prim[3 + i][lane] = vi.Sc[i];
-    prim[9][lane] = vi.beta_x;
-    for (int i = 0; i < 3; ++i) prim[10 + i][lane] = __ldg(sc.rgb + i * sc.P + p);
+    if (!vi.valid) cull_below = INFINITY;  // a record of an invalid kernel is never drawn
+    for (int i = 0; i < 3; ++i) cp.mx[i] = in.mx[i];
+    for (int k = 0; k < C; ++k) {
+      cp.mq[k] = in.mq[k];
+      cp.rl[k] = __frcp_rn(vi.Lh[tri(k, k)]);
+      cp.b8[k] = 8.0f * vi.beta_q[k];
+      for (int m = 0; m < k; ++m) cp.lo[k * (k - 1) / 2 + m] = vi.Lh[tri(k, m)];
+    }
+    cp.below = cull_below - 0.01f;
+    for (int i = 0; i < 3; ++i) prim[F::kMx + i][lane] = in.mx[i];
+    for (int i = 0; i < C; ++i) prim[F::kMq + i][lane] = in.mq[i];
+    for (int i = 0; i < C * (C + 1) / 2; ++i) prim[F::kLh + i][lane] = vi.Lh[i];
+    for (int i = 0; i < 3; ++i)
+      for (int k = 0; k < C; ++k) prim[F::kW3 + i * C + k][lane] = vi.W3[i][k];
+    for (int i = 0; i < C; ++i) prim[F::kBq + i][lane] = vi.beta_q[i];
+    prim[F::kO][lane] = in.o;
+    for (int i = 0; i < 6; ++i) prim[F::kSc + i][lane] = vi.Sc[i];
+    prim[F::kBx][lane] = vi.beta_x;
+    for (int i = 0; i < 3; ++i) prim[F::kRgb + i][lane] = __ldg(sc.rgb + i * sc.P + p);
+    prim[F::kBelow][lane] = cull_below;
   }
   __syncwarp();
-  // projects queue entry j (any lane may take any entry)
-  auto project = [&](int j) {
-    const uint32_t r = qr[j], kk = qk[j];
-    const int k = (int)(kk & 0xffffu), owner = (int)(kk >> 16);
-    float mx[3], Sc[6];
+  // queue entry j through the rule set (any lane may take any entry)
+  auto take = [&](int j) {
+    const uint32_t e = queue[j];
+    const int k = (int)(e & 0xffffu), owner = (int)(e >> 16);
+    const ViewDev& v = s_views[k];
+    const uint32_t r = v.rec_off + p0 + (uint32_t)owner;
+    PrimIn<C> in;
+    PrimVI<C> vi;
+    for (int i = 0; i < 3; ++i) in.mx[i] = prim[F::kMx + i][owner];
+    for (int i = 0; i < C; ++i) in.mq[i] = prim[F::kMq + i][owner];
+    for (int i = 0; i < C * (C + 1) / 2; ++i) vi.Lh[i] = prim[F::kLh + i][owner];
+    for (int i = 0; i < 3; ++i)
+      for (int m = 0; m < C; ++m) vi.W3[i][m] = prim[F::kW3 + i * C + m][owner];
+    for (int i = 0; i < C; ++i) vi.beta_q[i] = prim[F::kBq + i][owner];
+    in.o = prim[F::kO][owner];
     ViewCond c;
-    for (int i = 0; i < 3; ++i) {
-      mx[i] = prim[i][owner];
-      c.shift[i] = qf[i][j];
-      c.mc[i] = mx[i] + c.shift[i];
+    view_condition<C>(in, vi, v, c, prim[F::kBelow][owner]);
+    // an invalid kernel's bound is infinite (as is that of an opacity of zero, and
+    // one below zero has none: neither reaches alpha_min)
+    if (!view_candidate(prim[F::kBelow][owner] < INFINITY, c, v, cfg)) {
+      tiles[r] = 0;
+      return;
     }
-    c.oq = qf[3][j];
-    for (int i = 0; i < 6; ++i) Sc[i] = prim[3 + i][owner];
-    const float beta_x = prim[9][owner];
+    float Sc[6];
+    for (int i = 0; i < 6; ++i) Sc[i] = prim[F::kSc + i][owner];
+    const float beta_x = prim[F::kBx][owner];
     ViewOut o;
-    view_project(mx, Sc, beta_x, true, c, s_views[k], cfg, o);
+    view_project(in.mx, Sc, beta_x, true, c, v, cfg, o);
     tiles[r] = o.tiles;
     if (o.valid) {
       atomicOr(&s_vis[w][k], 1u << owner);
@@ -177,45 +267,40 @@ __global__ void __launch_bounds__(256, 3) preprocess_queued_kernel(SceneDev sc, 
       rect[r] = make_uint2((uint32_t)o.tx0 | ((uint32_t)o.ty0 << 16), (uint32_t)o.tx1 | ((uint32_t)o.ty1 << 16));
       rec4[3 * (size_t)r + 0] = make_float4(o.mu_hi[0], o.mu_hi[1], o.mu_lo[0], o.mu_lo[1]);
       rec4[3 * (size_t)r + 1] = make_float4(o.conic[0], o.conic[1], o.conic[2], log2f(o.oq));
-      rec4[3 * (size_t)r + 2] = make_float4(beta_x, prim[10][owner], prim[11][owner], prim[12][owner]);
+      rec4[3 * (size_t)r + 2] =
+          make_float4(beta_x, prim[F::kRgb][owner], prim[F::kRgb + 1][owner], prim[F::kRgb + 2][owner]);
       atomicOr(&s_any[w], 1u << owner);
     }
   };
   int qn = 0;  // warp-uniform
-  for (int k = 0; k < vl.n; ++k) {
-    const ViewDev& v = s_views[k];
-    bool cand = false;
-    ViewCond c;
-    uint32_t r = 0;
-    if (live) {
-      view_condition<C>(in, vi, v, c, cull_below);
-      r = v.rec_off + (uint32_t)p;
-      cand = view_candidate(vi.valid, c, v, cfg);
-      if (!cand) tiles[r] = 0;
+  for (int k = 0; k <= vl.n; ++k) {
+    if (k < vl.n) {
+      const ViewDev& v = s_views[k];
+      bool cand = false;
+      if (live) {
+        float cam[3];  // the camera's centre, as view_condition forms it
+        for (int i = 0; i < 3; ++i) cam[i] = -((v.R[i] * v.t[0] + v.R[3 + i] * v.t[1]) + v.R[6 + i] * v.t[2]);
+        cand = !certain_cull<C>(cp, cam, v.time);
+        if (!cand) tiles[v.rec_off + (uint32_t)p] = 0;
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, cand);
+      if (cand) queue[qn + __popc(m & lt)] = (uint32_t)k | ((uint32_t)lane << 16);
+      qn += __popc(m);
+      __syncwarp();
     }
-    const unsigned m = __ballot_sync(0xffffffffu, cand);
-    if (cand) {
-      const int j = qn + __popc(m & lt);
-      qr[j] = r;
-      qk[j] = (uint32_t)k | ((uint32_t)lane << 16);
-      for (int i = 0; i < 3; ++i) qf[i][j] = c.shift[i];
-      qf[3][j] = c.oq;
-    }
-    qn += __popc(m);
-    __syncwarp();
-    if (qn >= 32) {  // the 32 newest entries, one per lane
-      project(qn - 32 + lane);
-      qn -= 32;
+    // the 32 newest entries, one per lane; after the last view, the rest
+    if (qn >= 32 || (k == vl.n && qn > 0)) {
+      const int n = min(qn, 32);
+      if (lane < n) take(qn - n + lane);
+      qn -= n;
       __syncwarp();
     }
   }
-  if (lane < qn) project(lane);
   __syncwarp();
   // the warp's visibility mask word of each view (its primitives start at a
   // multiple of 32)
-  const int64_t p0 = p - lane;
-  if (p0 < sc.P)
-    for (int k = lane; k < vl.n; k += 32) vis_mask[s_views[k].mask_off + (uint32_t)(p0 >> 5)] = s_vis[w][k];
+  if ((int64_t)p0 < sc.P)
+    for (int k = lane; k < vl.n; k += 32) vis_mask[s_views[k].mask_off + (p0 >> 5)] = s_vis[w][k];
   // scenes with several views: the primitives some view sees, listed for the
   // parameter backward (one add per warp)
   const bool any = live && ((s_any[w] >> lane) & 1u);
@@ -256,7 +341,7 @@ cudaError_t launch_preprocess(const SceneDev& sc, const ViewList& vl, const View
     const cudaError_t e = prepare_queued();
     if (e != cudaSuccess) return e;
   }
-  const int threads = 256;
+  const int threads = sc.N > 3 ? kQThreads : 256;
   const unsigned blocks = (unsigned)((sc.P + threads - 1) / threads);
   const size_t smem = sizeof(ViewDev) * vl.n;
   float4* rec4 = (float4*)(ws + L.rec4);

@@ -320,6 +320,42 @@ def test_split_long_lists(make):
         assert (last > 2048).sum() > 50 and (last <= 2048).sum() > 50
 
 
+@pytest.mark.parametrize("N", [4, 6, 7])
+@pytest.mark.parametrize("P,n_views", [(127, 2), (20011, 5), (400, 70)])
+def test_query_cull_at_extremes(N, P, n_views):
+    """The cheap test that spares most records their exact conditioning culls
+    none that the rule set draws, and the queue behind it loses none: which
+    records are drawn, bit for bit against the oracle, over query scales from
+    1e-3 to 20, strongly correlated query blocks, Beta exponents from e^-8 to
+    e^8, opacities of 0, 1, about alpha_min and between, a query mean that
+    equals a view's time, and a primitive at a camera's centre."""
+    rng = np.random.default_rng(N * 1000 + P)
+    times = list(rng.uniform(0.0, 1.0, n_views))
+    sc = S.make_scene(N, N, P, means="clusters", extent=2.0, n_clusters=8, ang_scale=(1e-3, 20.0),
+                      time_scale=(1e-3, 20.0), lqx_amp=2.0, lq_amp=3.0, rng=rng)
+    views = S.sphere_views(rng, n_views, 5.0, 96, 80, hemisphere=True, times=times)
+    b = sc.plane("b")
+    b[1:] = rng.uniform(-8.0, 8.0, b[1:].shape).astype(np.float32)
+    op = sc.plane("opacity")[0]
+    kind = rng.integers(0, 6, P)
+    op[kind == 0], op[kind == 1] = 0.0, 1.0
+    op[kind == 2] = np.float32(1.0 / 255.0) * (1.0 + rng.uniform(-1e-6, 1e-6, (kind == 2).sum())).astype(np.float32)
+    if N in (4, 7):
+        sc.plane("mean_q")[0][:P // 3] = np.float32(views[0].time)
+    sc.plane("mean_x")[:, 0] = (-views[0].R.astype(np.float64).T @ views[0].t).astype(np.float32)
+    orc = R64.Oracle([sc], views, S.RasterConfig())
+    gpu = gpu_forward([sc], views, S.RasterConfig())
+    drawn = 0
+    for vi, pre in enumerate(orc.pre32):
+        o = int(orc.rec_off[vi])
+        tiles = gpu["tiles"][o:o + P].astype(np.int64)
+        assert np.array_equal(tiles, pre["tiles_touched"]), f"view {vi}"
+        v = pre["valid"]
+        assert np.array_equal(gpu["keys"][o:o + P][v], pre["depth_bits"][v])
+        drawn += int(v.sum())
+    assert drawn > 0
+
+
 @pytest.mark.parametrize("n_views,N", [(40, 6), (256, 7), (40, 3)])
 def test_many_views_of_one_scene(n_views, N):
     """More views than one 32-view mask of the parameter backward, up to the
