@@ -22,7 +22,9 @@
 //      many entries, and
 //   5. merge: one CTA per such list merges its sorted chunks pairwise in
 //      rounds (merge path: each thread an equal share of the outputs), in
-//      shared memory up to kMergeSeg entries, then in global memory.
+//      shared memory up to kMergeSeg entries, then in global memory; with
+//      split lists, where few lists are that long, a CTA per kMergeSeg
+//      entries, and a join by rank.
 // A record meets a tile once, so the keys of a tile are distinct and the
 // result does not depend on the bucket order: it is the order a stable
 // sort by (tile, depth) of the records in index order gives.
@@ -664,6 +666,9 @@ __global__ void __launch_bounds__(kTsW * 32, 8) tile_sort_kernel(const uint2* __
 // ---------------------------------------------------------------- merge
 
 constexpr int kMgT = 512;  // threads of a merge CTA
+// chunks of long lists up to which split-list problems join segments by rank
+// (about one wave of merge CTAs, of kMergeSeg entries each)
+constexpr uint32_t kJoinChunks = 2048;
 
 // Merges the sorted runs A = src[a0, a0 + na) and B = src[b0, b0 + nb)
 // (distinct keys) into dst[o0, o0 + na + nb), writing only the outputs
@@ -796,12 +801,13 @@ __global__ void __launch_bounds__(kMgT, 2) tile_merge_kernel(const uint2* __rest
                                                           unsigned long long* __restrict__ chunk64,
                                                           unsigned long long* __restrict__ tmp64,
                                                           uint32_t* __restrict__ out, Header* hdr,
-                                                          TileDescArgs D) {
+                                                          TileDescArgs D, bool join) {
   wait_prior_grid();
   make_tile_descs(D, tstart);
   __shared__ unsigned long long s_seg[kMergeSeg];
   __shared__ uint32_t s_it;
   const uint32_t n_long = hdr->n_long;
+  join = join && n_long <= kJoinChunks;
   for (;;) {
     // the next chunk item, from a counter: the CTAs stay busy however the
     // long lists fall among them; a list's first chunk stands for the list
@@ -811,8 +817,17 @@ __global__ void __launch_bounds__(kMgT, 2) tile_merge_kernel(const uint2* __rest
     const uint32_t it = s_it;
     if (it >= n_long) break;
     const uint2 item = items[it];
-    if (item.y != 0) continue;  // uniform over the block
+    if (item.y != 0 && !join) continue;  // uniform over the block
     const uint32_t s = tstart[item.x], L = tstart[item.x + 1] - s;
+    if (join && L > kMergeSeg) {  // one segment; tile_join_kernel does the rest
+      if (item.y % (kMergeSeg / kSortChunk) != 0) continue;
+      const uint32_t s0 = item.y * kSortChunk, n = min(kMergeSeg, L - s0);
+      merge_segment(chunk64 + s + s0, n, s_seg);
+      for (uint32_t i = threadIdx.x; i < n; i += kMgT) chunk64[s + s0 + i] = s_seg[i];
+      __syncthreads();  // the segment buffer is free for the block's next item
+      continue;
+    }
+    if (item.y != 0) continue;
     if (L <= kMergeSeg) {
       merge_segment(chunk64 + s, L, s_seg);
       for (uint32_t i = threadIdx.x; i < L; i += kMgT) out[s + i] = (uint32_t)s_seg[i];
@@ -844,6 +859,61 @@ __global__ void __launch_bounds__(kMgT, 2) tile_merge_kernel(const uint2* __rest
     }
     for (uint32_t i = threadIdx.x; i < L; i += kMgT) out[s + i] = (uint32_t)src[i];
     __syncthreads();
+  }
+}
+
+// Joins the sorted segments of lists over kMergeSeg entries where these are
+// few: every entry's place is its place in its own segment plus, by bisection,
+// the number of smaller keys in each other segment.  That is more work than
+// merging in rounds (12 loads per entry and other segment) but none of it
+// waits on any other, over as many CTAs as there are chunks, where the rounds
+// run on one CTA per list: two lists of 29,000 and two of 7,700 entries took
+// 191 us so, 23 us by segments and 21 in this kernel.  With more chunks than
+// kJoinChunks the lists keep the CTAs busy and the rounds' fewer loads win.
+__global__ void __launch_bounds__(kMgT) tile_join_kernel(const uint2* __restrict__ items,
+                                                         const uint32_t* __restrict__ tstart,
+                                                         const unsigned long long* __restrict__ chunk64,
+                                                         uint32_t* __restrict__ out, const Header* hdr) {
+  wait_prior_grid();
+  static_assert(kMgT == kSortChunk, "an entry of a chunk per thread");
+  const uint32_t n_long = hdr->n_long;
+  if (n_long > kJoinChunks) return;
+  for (uint32_t it = blockIdx.x; it < n_long; it += gridDim.x) {
+    const uint2 item = items[it];
+    const uint32_t s = tstart[item.x], L = tstart[item.x + 1] - s;
+    const uint32_t i = item.y * kSortChunk + threadIdx.x;
+    if (L <= kMergeSeg || i >= L) continue;
+    const unsigned long long* list = chunk64 + s;
+    const unsigned long long x = list[i];
+    const uint32_t own = i / kMergeSeg, n_seg = (L + kMergeSeg - 1) / kMergeSeg;
+    uint32_t rank = i - own * kMergeSeg;
+    constexpr int J = 4;  // bisections in flight
+    for (uint32_t j0 = 0; j0 < n_seg; j0 += J) {
+      uint32_t lo[J], n[J];
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
+        const uint32_t seg = j0 + j;
+        lo[j] = seg * kMergeSeg;
+        n[j] = seg < n_seg && seg != own ? min(kMergeSeg, L - lo[j]) : 0u;
+      }
+      // lower_bound by halving: after each step the n[j] entries from lo[j] on
+      // hold the border, at most kMergeSeg = 2^12 of them: 13 steps
+#pragma unroll 1
+      for (int step = 0; step < 13; ++step) {
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+          const uint32_t half = n[j] >> 1;
+          if (n[j] == 0) continue;
+          const bool below = list[lo[j] + half] < x;
+          lo[j] = below ? lo[j] + half + 1 : lo[j];
+          n[j] = below ? n[j] - half - 1 : half;
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < J; ++j)
+        if (j0 + j < n_seg && j0 + j != own) rank += lo[j] - (j0 + j) * kMergeSeg;
+    }
+    out[s + rank] = (uint32_t)x;  // the ranks are a permutation of 0 .. L - 1
   }
 }
 
@@ -915,11 +985,17 @@ cudaError_t launch_bin_sort(const Layout& L, const CfgDev& cfg, char* ws, cudaSt
   uint32_t* out = (uint32_t*)(ws + L.ivals);
   unsigned long long* chunk64 = (unsigned long long*)(ws + L.chunk64);
   const uint32_t ts_blocks = (L.max_items + kTsW - 1) / kTsW;
+  // problems made for long lists (UBS_FLAG_SPLIT_LISTS) launch the join too; for
+  // the others a launch more would cost what it could save
+  const bool join = (cfg.flags & kFlagSplit) != 0;
   launch_dependent(tile_sort_kernel, dim3(ts_blocks < kSortGrid ? ts_blocks : kSortGrid), dim3(kTsW * 32), 0, st,
                    (const uint2*)items, (const uint32_t*)tstart, (const uint32_t*)(ws + L.key), L.R,
                    (const uint32_t*)bucket, out, chunk64, hdr);
   launch_dependent(tile_merge_kernel, dim3(kMergeGrid), dim3(kMgT), 0, st, (const uint2*)items,
-                   (const uint32_t*)tstart, chunk64, (unsigned long long*)(ws + L.tmp64), out, hdr, D);
+                   (const uint32_t*)tstart, chunk64, (unsigned long long*)(ws + L.tmp64), out, hdr, D, join);
+  if (join)
+    launch_dependent(tile_join_kernel, dim3(kMergeGrid), dim3(kMgT), 0, st, (const uint2*)items,
+                     (const uint32_t*)tstart, (const unsigned long long*)chunk64, out, (const Header*)hdr);
   return cudaGetLastError();
 }
 

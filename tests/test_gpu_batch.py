@@ -212,3 +212,30 @@ def test_split_segments_at_their_edges(tile, n, cap):
     assert (got[True][0] - got[False][0]).abs().max() <= 1e-5
     worst = ((got[True][1] - got[False][1]).abs().amax(1) / got[False][1].abs().amax(1).clamp(min=1e-30)).max()
     assert worst <= 1e-3, float(worst)
+
+
+@pytest.mark.parametrize("n", [4096, 4097, 8192, 8193, 20000])
+def test_long_lists_joined_by_rank(n):
+    """Lists at and around the 4096 entries of one sorted segment, in the
+    split form (segments sorted by separate CTAs and joined by rank) and the
+    other (merged by one CTA): the same lists, bit for bit, and in the order of
+    (depth, record); with many records at one depth."""
+    rng = np.random.default_rng(n)
+    sc = S.make_scene(n, 3, n, scale_range=(0.02, 0.05), rng=rng)
+    sc.plane("mean_x")[:] = (0.0005 * rng.uniform(-1.0, 1.0, (3, n))).astype(np.float32)
+    sc.plane("mean_x")[2] = rng.choice(np.linspace(-0.5, 0.5, 97).astype(np.float32), n)
+    v = S.make_view(np.eye(3), np.array([0.0, 0.0, 4.0]), 75, 71)
+    lists = []
+    for split in (False, True):
+        r = raster.Rasterizer([raster.DeviceScene.from_scene(sc, device="cuda")], [v], S.RasterConfig(split_lists=split),
+                              device="cuda")
+        r.forward(check=True)
+        k = int(r.status().instances)
+        lists.append((r.export(U.EXPORT_TILE_START).clone(), r.export(U.EXPORT_INSTANCES)[:k].clone()))
+        keys = r.export(U.EXPORT_KEYS).cpu().numpy().view(np.uint32)
+    assert all(torch.equal(a, b) for a, b in zip(*lists))
+    start, inst = (t.cpu().numpy().view(np.uint32).astype(np.int64) for t in lists[1])
+    assert np.diff(start).max() >= 4096
+    for s, e in zip(start[:-1], start[1:]):
+        order = inst[s:e]
+        assert np.array_equal(order, order[np.lexsort((order, keys[order]))]) and np.unique(order).size == order.size
