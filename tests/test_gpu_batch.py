@@ -239,3 +239,25 @@ def test_long_lists_joined_by_rank(n):
     for s, e in zip(start[:-1], start[1:]):
         order = inst[s:e]
         assert np.array_equal(order, order[np.lexsort((order, keys[order]))]) and np.unique(order).size == order.size
+
+
+@pytest.mark.parametrize("tile", [(8, 8), (16, 16), (16, 32), (32, 32)])
+def test_few_tiles_match_many(tile):
+    """A view alone (few tiles: the forward that evaluates four entries ahead)
+    and the same view among enough copies to fill the GPU (the general form):
+    images, final T and last contributors bit for bit."""
+    rng = np.random.default_rng(tile[0] + tile[1])
+    sc = S.make_scene(9, 3, 3001, scale_range=(0.02, 0.2), rng=rng)
+    v = S.make_view(np.eye(3), np.array([0.0, 0.0, 3.0]), 101, 77)
+    tiles = -(-v.width // tile[0]) * -(-v.height // tile[1])
+    warps = tiles * tile[0] * tile[1] // 64
+    n = 152 * 4 * 2 // warps + 1
+    assert warps <= 152 * 4 * 2 < n * warps and n <= 256
+    got = []
+    for k in (1, n):
+        r = raster.Rasterizer([raster.DeviceScene.from_scene(sc, device="cuda")], [v] * k,
+                              S.RasterConfig(tile_w=tile[0], tile_h=tile[1]), device="cuda")
+        r.forward(check=True)
+        px = v.width * v.height
+        got.append((r.image[:3 * px].clone(), r.export(U.EXPORT_FINAL_T)[:px].clone(), r.export(U.EXPORT_LAST)[:px].clone()))
+    assert all(torch.equal(a, b) for a, b in zip(*got))
