@@ -163,7 +163,8 @@ __device__ __forceinline__ uint32_t bucket_add(uint32_t* s, int b) {
 // before it (totals, complete over every block), and each block takes its
 // part of that range from the bucket's cursor.  Returns the position, ~0
 // where b < 0.  Block-uniform call (every thread).
-template <int NT>
+// With ONE block, its own counts are the totals and its parts the ranges.
+template <int NT, bool ONE = false>
 __device__ __forceinline__ uint32_t bucket_place(const uint32_t* __restrict__ totals, uint32_t* __restrict__ cursors,
                                                  int b, uint32_t* s_n, uint32_t* s_base) {
   for (int i = threadIdx.x; i < kOrdBuckets; i += NT) s_n[i] = 0;
@@ -177,7 +178,7 @@ __device__ __forceinline__ uint32_t bucket_place(const uint32_t* __restrict__ to
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
       const uint32_t i = lane * PER + j;
-      tot[j] = i < (uint32_t)kOrdBuckets ? totals[i] : 0u;
+      tot[j] = i < (uint32_t)kOrdBuckets ? (ONE ? s_n[i] : totals[i]) : 0u;
       sum += tot[j];
     }
     uint32_t incl = sum;
@@ -190,7 +191,7 @@ __device__ __forceinline__ uint32_t bucket_place(const uint32_t* __restrict__ to
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
       const uint32_t i = lane * PER + j;
-      if (i < (uint32_t)kOrdBuckets && s_n[i]) s_base[i] = start + atomicAdd(cursors + i, s_n[i]);
+      if (i < (uint32_t)kOrdBuckets && s_n[i]) s_base[i] = ONE ? start : start + atomicAdd(cursors + i, s_n[i]);
       start += tot[j];
     }
   }
@@ -292,7 +293,9 @@ __global__ void __launch_bounds__(kScT) scan_mid_kernel(const ScanPart* __restri
 // order.  With few blocks (pre null) a block sums the earlier blocks' parts
 // itself; else it reads the prefixes and totals of scan_mid_kernel.  Block
 // 0 records the totals (and a capacity overflow, after which every list is
-// empty and there is no item).
+// empty and there is no item).  With ONE block (up to kScanTiles tiles) the
+// totals are its own and there is no first pass: 3 us and a launch less.
+template <bool ONE>
 __global__ void __launch_bounds__(kScT) scan_place_kernel(const uint32_t* __restrict__ tcount, uint32_t NT,
                                                           uint32_t cap, const ScanPart* __restrict__ part, uint32_t nb,
                                                           const ScanPart* __restrict__ pre,
@@ -306,7 +309,7 @@ __global__ void __launch_bounds__(kScT) scan_place_kernel(const uint32_t* __rest
   __shared__ uint32_t s_w[kScT / 32 + 1];
   __shared__ uint32_t s_n[kOrdBuckets], s_base[kOrdBuckets];
   __shared__ ScanPart s_pt[2];
-  if (threadIdx.x < 32) {
+  if (!ONE && threadIdx.x < 32) {
     // the parts before this block (P) and of all blocks (T): one warp
     ScanPart P{0ull, 0u, 0u}, T{0ull, 0u, 0u};
     if (pre) {
@@ -331,8 +334,8 @@ __global__ void __launch_bounds__(kScT) scan_place_kernel(const uint32_t* __rest
     if (threadIdx.x == 0) s_pt[0] = P, s_pt[1] = T;
   }
   __syncthreads();
-  const ScanPart P = s_pt[0], T = s_pt[1];
-  const bool over = T.inst > cap;
+  ScanPart P{0ull, 0u, 0u}, T{0ull, 0u, 0u};
+  if (!ONE) P = s_pt[0], T = s_pt[1];
   const uint32_t t = blockIdx.x * kScT + threadIdx.x;
   uint32_t c[kTileSub];
   const uint32_t n = load_tile_counts(tcount, t, NT, c);
@@ -342,8 +345,10 @@ __global__ void __launch_bounds__(kScT) scan_place_kernel(const uint32_t* __rest
   block_excl_scan2<kScT>((unsigned long long)n, nl, ei, el, bi, bl, s_w64, s_w);
   // the short lists' items, after every long list's chunks, longest first
   const bool is_short = t < NT && n > 0 && n <= kSortChunk;
-  const uint32_t ps = bucket_place<kScT>(order_count + 2 * kOrdBuckets, order_count + 3 * kOrdBuckets,
-                                         is_short ? length_bucket(n) : -1, s_n, s_base);
+  const uint32_t ps = bucket_place<kScT, ONE>(order_count + 2 * kOrdBuckets, order_count + 3 * kOrdBuckets,
+                                              is_short ? length_bucket(n) : -1, s_n, s_base);
+  if (ONE) T = ScanPart{bi, bl, (uint32_t)__syncthreads_count(is_short)};
+  const bool over = T.inst > cap;
   if (t < NT) {
     uint32_t run = over ? 0u : (uint32_t)(P.inst + ei);
     tstart[t] = run;
@@ -367,7 +372,7 @@ __global__ void __launch_bounds__(kScT) scan_place_kernel(const uint32_t* __rest
     hdr->n_items = over ? 0u : T.n_long + T.n_short;
     if (over) set_status(hdr, kDevCapacity);
   }
-  if (order && !over && T.inst >= (unsigned long long)kOrdDense * NT) {  // uniform over the block
+  if (!ONE && order && !over && T.inst >= (unsigned long long)kOrdDense * NT) {  // uniform over the block
     const uint32_t pos = bucket_place<kScT>(order_count, order_count + kOrdBuckets, t < NT ? length_bucket(n) : -1,
                                             s_n, s_base);
     if (t < NT && pos < NT) order[pos] = t;  // pos < NT holds: the totals count every tile
@@ -966,17 +971,25 @@ cudaError_t launch_bin_sort(const Layout& L, const CfgDev& cfg, char* ws, cudaSt
   static_assert(kVisBlocks >= kScatGrid, "a visible-record count per walk block");
   const uint32_t nb = L.n_scan_blocks;
   ScanPart* part = (ScanPart*)(ws + L.scan_part);
-  launch_dependent(scan_part_kernel, dim3(nb), dim3(kScT), 0, st, tcount, L.NT, part,
-                   order_count, order != nullptr);
-  ScanPart* pre = nullptr;
-  ScanPart* tot = nullptr;
-  if (nb > kFusePrefixMax) {
-    pre = part + nb;
-    tot = part + 2 * nb;
-    launch_dependent(scan_mid_kernel, dim3(1), dim3(kScT), 0, st, (const ScanPart*)part, nb, pre, tot);
+  static_assert(kOrdMinTiles >= kScanTiles, "no tile order is made by one block");
+  if (nb == 1) {
+    launch_dependent(scan_place_kernel<true>, dim3(1), dim3(kScT), 0, st, tcount, L.NT, L.cap, (const ScanPart*)part,
+                     nb, (const ScanPart*)nullptr, (const ScanPart*)nullptr, hdr, tstart, cursor, items, order_count,
+                     order);
+  } else {
+    launch_dependent(scan_part_kernel, dim3(nb), dim3(kScT), 0, st, tcount, L.NT, part, order_count,
+                     order != nullptr);
+    ScanPart* pre = nullptr;
+    ScanPart* tot = nullptr;
+    if (nb > kFusePrefixMax) {
+      pre = part + nb;
+      tot = part + 2 * nb;
+      launch_dependent(scan_mid_kernel, dim3(1), dim3(kScT), 0, st, (const ScanPart*)part, nb, pre, tot);
+    }
+    launch_dependent(scan_place_kernel<false>, dim3(nb), dim3(kScT), 0, st, tcount, L.NT, L.cap,
+                     (const ScanPart*)part, nb, (const ScanPart*)pre, (const ScanPart*)tot, hdr, tstart, cursor,
+                     items, order_count, order);
   }
-  launch_dependent(scan_place_kernel, dim3(nb), dim3(kScT), 0, st, tcount, L.NT, L.cap, (const ScanPart*)part, nb,
-                   (const ScanPart*)pre, (const ScanPart*)tot, hdr, tstart, cursor, items, order_count, order);
   uint32_t* bucket = (uint32_t*)(ws + L.bucket);
   launch_dependent(scatter_kernel, walk_grid, dim3(kScatT), 0, st, (const uint32_t*)(ws + L.tiles),
                    (const uint2*)(ws + L.rect), (const uint32_t*)(ws + L.vis_mask), L.mask_words, chunk,
