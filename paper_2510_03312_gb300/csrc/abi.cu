@@ -267,6 +267,8 @@ ubs_status ubs_preprocess(const ubs_problem* pr, void* ws, size_t ws_bytes, cuda
   // view table: per-view constants, tile/record/pixel/mask offsets
   ViewDev* views = (ViewDev*)(w + L.views);
   uint32_t tile_off = 0, rec_off = 0, pix_off = 0, mask_off = 0;
+  OneView one;
+  memset(&one, 0, sizeof(one));
   for (int c0 = 0; c0 < L.V; c0 += kUploadChunk) {
     ViewChunk chunk;
     memset(&chunk, 0, sizeof(chunk));
@@ -296,6 +298,11 @@ ubs_status ubs_preprocess(const ubs_problem* pr, void* ws, size_t ws_bytes, cuda
       mask_off += (uint32_t)((pr->scenes[v.scene_id].P + 31) / 32);
     }
     static_assert(sizeof(Header) % 4 == 0, "the header is zeroed by words");
+    if (L.V == 1 && pr->scenes[pr->views[0].scene_id].P > 0) {  // a launch less: the preprocess kernel takes it along
+      one = OneView{chunk.v[0], views, (uint32_t*)(w + L.header), (uint32_t)(sizeof(Header) / 4),
+                    (uint32_t*)(w + L.act_count), L.S, 1};
+      break;
+    }
     upload_views_kernel<<<1, kUploadChunk, 0, stream>>>(chunk, n, views + c0,
                                                          c0 == 0 ? (uint32_t*)(w + L.header) : nullptr,
                                                          (uint32_t)(sizeof(Header) / 4), (uint32_t*)(w + L.act_count),
@@ -317,7 +324,7 @@ ubs_status ubs_preprocess(const ubs_problem* pr, void* ws, size_t ws_bytes, cuda
     uint32_t* zero = launches && !zeroed ? (uint32_t*)(w + L.tcount) : nullptr;
     zeroed = zeroed || launches;
     e = launch_preprocess(scene_dev(pr->scenes[s]), vl, views, cfg, L, w, (uint32_t*)(w + L.act_list) + act_off,
-                          (uint32_t*)(w + L.act_count) + s, zero, zero ? nzero : 0u, stream);
+                          (uint32_t*)(w + L.act_count) + s, zero, zero ? nzero : 0u, one, stream);
     act_off += (uint64_t)pr->scenes[s].P;
     if (e != cudaSuccess) return UBS_ERR_CUDA;
   }

@@ -106,13 +106,26 @@ struct ViewList {
   int16_t idx[kMaxViews];
 };
 
+// With one view, the first kernel gets it as an argument (on) and, in its first
+// block, writes the view table and zeroes the status header and the scenes'
+// counts of drawn primitives, which upload_views_kernel does for several.
+struct OneView {
+  ViewDev v;
+  ViewDev* dst;
+  uint32_t* hdr;
+  uint32_t hdr_words;
+  uint32_t* act_count;
+  int32_t S;
+  int32_t on;
+};
+
 // act_list/act_count: the scene's list of primitives visible in some view
 // (appended by preprocess, read by the parameter backward)
 // zero/nzero: words the launch zeroes besides its own work (the binning's
 // counters), or none
 cudaError_t launch_preprocess(const SceneDev& sc, const ViewList& vl, const ViewDev* views, const CfgDev& cfg,
                               const Layout& L, char* ws, uint32_t* act_list, uint32_t* act_count, uint32_t* zero,
-                              uint32_t nzero, cudaStream_t st);
+                              uint32_t nzero, const OneView& one, cudaStream_t st);
 
 // count, scan (ranges), scatter, per-tile sort and merge; leaves the sorted
 // instance records in the buffer reported by sorted_instances()

@@ -38,17 +38,33 @@ __device__ __forceinline__ void zero_words(uint32_t* __restrict__ zero, uint32_t
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) zero[i] = 0;
 }
 
+// The first block's part for a problem of one view (see OneView).
+__device__ __forceinline__ void start_one_view(const OneView& one) {
+  if (!one.on || blockIdx.x != 0) return;
+  const uint32_t n = sizeof(ViewDev) / 4;
+  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x)
+    reinterpret_cast<uint32_t*>(one.dst)[i] = reinterpret_cast<const uint32_t*>(&one.v)[i];
+  for (uint32_t i = threadIdx.x; i < one.hdr_words; i += blockDim.x) one.hdr[i] = 0;
+  for (int i = threadIdx.x; i < one.S; i += blockDim.x) one.act_count[i] = 0;
+}
+
 template <int C>
 __global__ void __launch_bounds__(256) preprocess_kernel(SceneDev sc, ViewList vl, const ViewDev* __restrict__ views,
                                                          CfgDev cfg, float4* __restrict__ rec4,
                                                          uint32_t* __restrict__ key, uint32_t* __restrict__ tiles,
                                                          uint2* __restrict__ rect, uint32_t* __restrict__ vis_mask,
                                                          uint32_t* __restrict__ act_list, uint32_t* act_count,
-                                                         uint32_t* __restrict__ zero, uint32_t nzero) {
+                                                         uint32_t* __restrict__ zero, uint32_t nzero,
+                                                         const __grid_constant__ OneView one) {
   wait_prior_grid();
   zero_words(zero, nzero);
+  start_one_view(one);
   extern __shared__ ViewDev s_views[];
-  for (int i = threadIdx.x; i < vl.n; i += blockDim.x) s_views[i] = views[vl.idx[i]];
+  if (one.on) {
+    if (threadIdx.x == 0) s_views[0] = one.v;
+  } else {
+    for (int i = threadIdx.x; i < vl.n; i += blockDim.x) s_views[i] = views[vl.idx[i]];
+  }
   __syncthreads();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= sc.P) return;
@@ -241,15 +257,18 @@ template <int C>
 __global__ void __launch_bounds__(kOneThreads, 4) preprocess_one_view_kernel(
     SceneDev sc, ViewList vl, const ViewDev* __restrict__ views, CfgDev cfg, float4* __restrict__ rec4,
     uint32_t* __restrict__ key, uint32_t* __restrict__ tiles, uint2* __restrict__ rect,
-    uint32_t* __restrict__ vis_mask, uint32_t* __restrict__ zero, uint32_t nzero) {
+    uint32_t* __restrict__ vis_mask, uint32_t* __restrict__ zero, uint32_t nzero,
+    const __grid_constant__ OneView one) {
   wait_prior_grid();
   zero_words(zero, nzero);
+  start_one_view(one);
   __shared__ ViewDev s_view;
   __shared__ uint32_t s_vis[kOnePrims / 32], s_n;
   __shared__ uint16_t s_list[kOnePrims];
   if (threadIdx.x < sizeof(ViewDev) / 4)
     reinterpret_cast<uint32_t*>(&s_view)[threadIdx.x] =
-        reinterpret_cast<const uint32_t*>(views + vl.idx[0])[threadIdx.x];
+        one.on ? reinterpret_cast<const uint32_t*>(&one.v)[threadIdx.x]
+               : reinterpret_cast<const uint32_t*>(views + vl.idx[0])[threadIdx.x];
   if (threadIdx.x < kOnePrims / 32) s_vis[threadIdx.x] = 0;
   if (threadIdx.x == 0) s_n = 0;
   __syncthreads();
@@ -477,7 +496,7 @@ cudaError_t prepare_queued() {
 
 cudaError_t launch_preprocess(const SceneDev& sc, const ViewList& vl, const ViewDev* views, const CfgDev& cfg,
                               const Layout& L, char* ws, uint32_t* act_list, uint32_t* act_count, uint32_t* zero,
-                              uint32_t nzero, cudaStream_t st) {
+                              uint32_t nzero, const OneView& one, cudaStream_t st) {
   if (sc.P == 0 || vl.n == 0) return cudaSuccess;
   if (sc.N > 3) {
     const cudaError_t e = prepare_queued();
@@ -494,15 +513,15 @@ cudaError_t launch_preprocess(const SceneDev& sc, const ViewList& vl, const View
   if (sc.N > 3 && vl.n == 1) {
     const dim3 grid((unsigned)((sc.P + kOnePrims - 1) / kOnePrims)), block(kOneThreads);
     switch (sc.N) {
-      case 4: launch_dependent(preprocess_one_view_kernel<1>, grid, block, 0, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, zero, nzero); break;
-      case 6: launch_dependent(preprocess_one_view_kernel<3>, grid, block, 0, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, zero, nzero); break;
-      case 7: launch_dependent(preprocess_one_view_kernel<4>, grid, block, 0, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, zero, nzero); break;
+      case 4: launch_dependent(preprocess_one_view_kernel<1>, grid, block, 0, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, zero, nzero, one); break;
+      case 6: launch_dependent(preprocess_one_view_kernel<3>, grid, block, 0, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, zero, nzero, one); break;
+      case 7: launch_dependent(preprocess_one_view_kernel<4>, grid, block, 0, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, zero, nzero, one); break;
       default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
   }
   switch (sc.N) {
-    case 3: launch_dependent(preprocess_kernel<0>, dim3(blocks), dim3(threads), smem, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, act_list, act_count, zero, nzero); break;
+    case 3: launch_dependent(preprocess_kernel<0>, dim3(blocks), dim3(threads), smem, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, act_list, act_count, zero, nzero, one); break;
     case 4: launch_dependent(preprocess_queued_kernel<1>, dim3(blocks), dim3(threads), smem, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, act_list, act_count, zero, nzero); break;
     case 6: launch_dependent(preprocess_queued_kernel<3>, dim3(blocks), dim3(threads), smem, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, act_list, act_count, zero, nzero); break;
     case 7: launch_dependent(preprocess_queued_kernel<4>, dim3(blocks), dim3(threads), smem, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, act_list, act_count, zero, nzero); break;
