@@ -93,7 +93,7 @@ enum {
                               slot) that take tiles or 8x8 blocks from a counter in the same order,
                               instead of one CTA per tile or block; the results are the same */
   UBS_FLAG_SPLIT_LISTS = 16, /* tile lists longer than 2048 entries are split into segments of 128 to
-                               2048 entries (the shortest whose state the workspace holds)
+                               2048 entries (as short as their number and the workspace allow)
                                blended by separate CTAs and merged front to back with the over
                                operator (C = C_1 + T_1 C_2, T = T_1 T_2), walking a segment again
                                for the pixels whose transmittance falls below T_min inside it; the

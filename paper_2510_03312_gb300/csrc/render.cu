@@ -559,10 +559,12 @@ __global__ void __launch_bounds__(TW * TH / 2) render_fwd_few_kernel(FwdArgs A) 
 // and 0.4 us backward when few segments share an SM, so short segments win
 // (two tiles of 29,000 entries and two of 7,700 in a sparse 1600x1060 view:
 // forward 385 + resume 279 + backward 589 us with 2048 entries, 157 + 75 +
-// 224 with 512, 106 + 23 + 157 with 128).  The length is the
-// shortest for which the slots hold every segment: the long lists' sort
-// chunks (n_long, of kSortChunk entries) bound their number, and seg_safe
-// is one that always does.
+// 224 with 512, 106 + 23 + 157 with 128).  The length is the shortest for
+// which there are at most kSegTarget segments (with more the GPU is full, and
+// the many later segments of lists that end early only cost) and the slots
+// hold them all: the long lists' sort chunks (n_long, of kSortChunk entries)
+// bound their number, and seg_safe is a length for which they always do.
+constexpr uint32_t kSegTarget = 152 * 16;
 __global__ void __launch_bounds__(256) split_plan_kernel(const uint32_t* __restrict__ tstart, uint32_t NT,
                                                          uint4* __restrict__ split_list,
                                                          uint32_t* __restrict__ tile_split,
@@ -574,7 +576,10 @@ __global__ void __launch_bounds__(256) split_plan_kernel(const uint32_t* __restr
   wait_prior_grid();
   if (hdr->status != 0) return;
   uint32_t seg_len = seg_min;
-  while (seg_len < seg_safe && (uint64_t)hdr->n_long * (seg_len < kSortChunk ? kSortChunk / seg_len : 1u) > max_slots)
+  const uint64_t chunks = hdr->n_long;
+  while (seg_len < kSplitMin &&
+         (chunks * kSortChunk > (uint64_t)kSegTarget * seg_len ||
+          (seg_len < seg_safe && chunks * (seg_len < kSortChunk ? kSortChunk / seg_len : 1u) > max_slots)))
     seg_len *= 2;
   if (blockIdx.x == 0 && threadIdx.x == 0) hdr->ctr[kCtrSegLen] = seg_len;
   for (uint32_t g = blockIdx.x * 256 + threadIdx.x; g < NT; g += gridDim.x * 256) {
@@ -635,14 +640,17 @@ __global__ void __launch_bounds__(TW * TH / 2, (TW * TH / 2 >= 128 ? 1024 / (TW 
 // (the local walk stopped, or T T_k < T_min) is where the pixel's walk ends,
 // and that segment is walked again from the pixel's true T.
 //
-// Passes 1 and 3 give a CTA 32 pixels of a split tile, a pixel per lane, and
-// each of its kJoinW warps an equal run of the tile's segments: a walk over
-// all segments by one thread per pixel is bound by the latency of its loads
-// (226 segments: 50 and 112 us for the two passes; 14 and 12 us so).
+// Passes 1 and 3 give 32 pixels of a split tile, a pixel per lane, to up to
+// kJoinW warps, each an equal run of the tile's segments: a walk over all
+// segments by one thread per pixel is bound by the latency of its loads (226
+// segments: 50 and 112 us for the two passes; 14 and 12 us so).  Where the
+// segments are few, fewer warps share a group of pixels (join_warps: four
+// segments a warp), and the CTA takes several groups.
 constexpr int kJoinW = 8;
-// warp w's segments [k0, k1) of m, from segment `first`
-__device__ __forceinline__ void join_share(uint32_t first, uint32_t m, int w, uint32_t& k0, uint32_t& k1) {
-  const uint32_t n = m > first ? m - first : 0u, per = (n + kJoinW - 1) / kJoinW;
+__device__ __forceinline__ int join_warps(uint32_t m) { return m <= 5 ? 1 : m <= 9 ? 2 : m <= 17 ? 4 : kJoinW; }
+// the segments [k0, k1) of m, from segment `first`, of warp w of G
+__device__ __forceinline__ void join_share(uint32_t first, uint32_t m, int w, int G, uint32_t& k0, uint32_t& k1) {
+  const uint32_t n = m > first ? m - first : 0u, per = (n + G - 1) / G;
   k0 = min(m, first + w * per);
   k1 = min(m, k0 + per);
 }
@@ -661,20 +669,26 @@ __global__ void __launch_bounds__(32 * kJoinW) split_join_kernel(FwdArgs A) {
   wait_prior_grid();
   constexpr int TP = TW * TH, CPT = TP / 32;  // CTAs' shares per tile
   __shared__ float s_T[kJoinW][32];
-  __shared__ uint32_t s_last[kJoinW][32], s_end[32], s_fin[32];
+  __shared__ uint32_t s_last[kJoinW][32], s_end[kJoinW][32], s_fin[kJoinW][32];
   if (A.hdr->status != 0) return;
   const CfgDev& cfg = A.cfg;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t n_items = A.hdr->ctr[4] * CPT;
   for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
     const uint4 sp = A.split_list[it / CPT];
-    const uint32_t m = sp.z, px = (it % CPT) * 32 + lane;
+    const uint32_t m = sp.z;
+    const int G = join_warps(m), grp = w / G, wg = w % G;  // this warp's group of 32 pixels, and its place among the group's warps
+    const uint32_t group = (it % CPT) * (kJoinW / G) + grp;
+    if ((it % CPT) * (kJoinW / G) >= CPT) continue;  // uniform: the tile's groups are taken
+    const bool mine = group < CPT;                   // a tile of two groups may not fill the CTA
+    const uint32_t px = (mine ? group : 0u) * 32 + lane;
     float4* my = A.seg_c + (size_t)sp.y * TP + px;  // slot k: my[k TP], my_l[k TP]
     uint32_t* my_l = A.seg_l + (size_t)sp.y * TP + px;
     const float T0 = my[0].w;
     const uint32_t l0 = my_l[0];
     uint32_t k0, k1;
-    join_share(1, m, w, k0, k1);
+    join_share(1, m, wg, G, k0, k1);
+    if (!mine) k0 = k1 = 0;
     float T = 1.0f;
     uint32_t last = 0;  // with kSegEnded where a segment ended the pixel
 #pragma unroll 4
@@ -686,12 +700,12 @@ __global__ void __launch_bounds__(32 * kJoinW) split_join_kernel(FwdArgs A) {
     }
     s_T[w][lane] = T;
     s_last[w][lane] = last;
-    if (w == 0) s_end[lane] = (l0 & kSegEnded) ? 0u : m - 1;  // ended in the first segment, or outside the image
+    if (wg == 0) s_end[grp][lane] = (l0 & kSegEnded) ? 0u : m - 1;  // ended in the first segment, or outside the image
     __syncthreads();
     float T1 = T0;  // at the start of this run
     last = l0 & ~kSegEnded;
     bool on = (l0 & kSegEnded) == 0u;
-    for (int h = 0; h < w; ++h) {  // the runs before this one
+    for (int h = w - wg; h < w; ++h) {  // the runs before this one
       T1 = __fmul_rn(T1, s_T[h][lane]);
       const uint32_t l = s_last[h][lane];
       on = on && !(l & kSegEnded) && T1 >= cfg.tmin;
@@ -710,7 +724,7 @@ __global__ void __launch_bounds__(32 * kJoinW) split_join_kernel(FwdArgs A) {
       if (!on) continue;
       if ((l & kSegEnded) || Tk < cfg.tmin) {
         on = false;
-        s_end[lane] = k | kSegEnded;  // one warp's: no later run goes on
+        s_end[grp][lane] = k | kSegEnded;  // one warp's: no later run goes on
         my[(size_t)k * TP].w = Ts;
         my_l[(size_t)k * TP] = last;
         continue;
@@ -719,13 +733,13 @@ __global__ void __launch_bounds__(32 * kJoinW) split_join_kernel(FwdArgs A) {
       last = l ? l : last;
     }
     // the last contributor over the whole walk: of the last run that goes on
-    if (w == kJoinW - 1 && on) s_fin[lane] = last;
+    if (wg == G - 1 && on) s_fin[grp][lane] = last;
     __syncthreads();
-    if (w == 0) {
-      const uint32_t end = s_end[lane];
+    if (wg == 0 && mine) {
+      const uint32_t end = s_end[grp][lane];
       A.seg_end[(size_t)(it / CPT) * TP + px] = end;
       // with a walk that ends in a later segment, that segment's own counts
-      my_l[0] = end == m - 1 ? s_fin[lane] : l0 & ~kSegEnded;
+      my_l[0] = end == m - 1 ? s_fin[grp][lane] : l0 & ~kSegEnded;
     }
     __syncthreads();  // shared memory is free for the next share
   }
@@ -772,14 +786,18 @@ __global__ void __launch_bounds__(32 * kJoinW) split_finish_kernel(FwdArgs A) {
   const uint32_t n_items = A.hdr->ctr[4] * CPT;
   for (uint32_t it = blockIdx.x; it < n_items; it += gridDim.x) {
     const uint4 sp = A.split_list[it / CPT];
-    const uint32_t px = (it % CPT) * 32 + lane;
+    const int G = join_warps(sp.z), grp = w / G, wg = w % G;  // as in the join
+    const uint32_t group = (it % CPT) * (kJoinW / G) + grp;
+    if ((it % CPT) * (kJoinW / G) >= CPT) continue;
+    const bool mine = group < CPT;
+    const uint32_t px = (mine ? group : 0u) * 32 + lane;
     float4* my = A.seg_c + (size_t)sp.y * TP + px;
     const uint32_t* my_l = A.seg_l + (size_t)sp.y * TP + px;
     const uint32_t end = A.seg_end[(size_t)(it / CPT) * TP + px];
     const uint32_t kend = end & ~kSegEnded;  // the last segment that adds anything
     uint32_t k0, k1;
-    join_share(0, sp.z, w, k0, k1);
-    k1 = min(k1, kend + 1);
+    join_share(0, sp.z, wg, G, k0, k1);
+    k1 = mine ? min(k1, kend + 1) : 0u;
     float C0 = 0.0f, C1 = 0.0f, C2 = 0.0f;
 #pragma unroll 4
     for (uint32_t k = k0; k < k1; ++k) {
@@ -791,11 +809,11 @@ __global__ void __launch_bounds__(32 * kJoinW) split_finish_kernel(FwdArgs A) {
     const float T = my[(size_t)kend * TP].w;
     s_c[w][lane] = make_float4(C0, C1, C2, 0.0f);
     __syncthreads();
-    if (w == 0) {
+    if (wg == 0 && mine) {
       const Tile v = make_tile(A.desc[sp.x], A.tpix[sp.x]);
       const int x = v.x0 + (int)(px % TW), y = v.y0 + (int)(px / TW);
       if (x < v.W && y < v.H) {
-        for (int h = 1; h < kJoinW; ++h) {
+        for (int h = w + 1; h < w + G; ++h) {
           C0 += s_c[h][lane].x;
           C1 += s_c[h][lane].y;
           C2 += s_c[h][lane].z;
@@ -810,7 +828,7 @@ __global__ void __launch_bounds__(32 * kJoinW) split_finish_kernel(FwdArgs A) {
       }
     }
     float b0 = T * cfg.bg[0], b1 = T * cfg.bg[1], b2 = T * cfg.bg[2];
-    for (int h = kJoinW - 1; h > w; --h) {
+    for (int h = w - wg + G - 1; h > w; --h) {
       b0 += s_c[h][lane].x;
       b1 += s_c[h][lane].y;
       b2 += s_c[h][lane].z;
@@ -1215,10 +1233,14 @@ cudaError_t fwd_launch(const FwdArgs& args, const Layout& L, bool persistent, cu
 
 // Split lists: the plan (after zeroing its counters), the grid of extra
 // segments and tiles, and the merge of the split tiles.  The grids over
-// segments, slots and split tiles are sized by the capacity's bounds, which
-// the lists rarely come near, up to a few CTAs per SM; beyond that they loop.
+// segments, slots and pixel groups hold a few CTAs per SM, or as many as
+// segments of kSplitMin entries would need (a CTA each, where the lists are
+// many), and loop over what the capacity's bounds allow beyond.
 constexpr uint32_t kSplitGrid = 152 * 8;
-inline uint32_t split_grid(uint32_t n) { return n < kSplitGrid ? n : kSplitGrid; }
+inline uint32_t split_grid(uint32_t n, uint32_t least) {
+  const uint32_t g = least > kSplitGrid ? least : kSplitGrid;
+  return n < g ? n : g;
+}
 
 template <int TW, int TH>
 cudaError_t fwd_split(const FwdArgs& args, const Layout& L, char* ws, cudaStream_t st) {
@@ -1235,7 +1257,7 @@ cudaError_t fwd_split(const FwdArgs& args, const Layout& L, char* ws, cudaStream
   if (e != cudaSuccess) return e;
   e = launch_dependent(render_fwd_kernel<TW, TH, false, true>, dim3(args.max_extra + L.NT), dim3(NT), 0, st, args);
   if (e != cudaSuccess) return e;
-  const dim3 shares(split_grid(L.seg_max_split * (TW * TH / 32)));
+  const dim3 shares(split_grid(L.seg_max_split * (TW * TH / 32), L.seg_max_split));
   e = launch_dependent(split_join_kernel<TW, TH>, shares, dim3(32 * kJoinW), 0, st, args);
   if (e != cudaSuccess) return e;
   e = launch_dependent(split_resume_kernel<TW, TH>, dim3(args.max_slots), dim3(NT), 0, st, args);
@@ -1272,8 +1294,8 @@ cudaError_t fwd_t(const Layout& L, const CfgDev& cfg, char* ws, float* image, cu
   a.seg_c = split ? (float4*)(ws + L.seg_c) : nullptr;
   a.seg_l = split ? (uint32_t*)(ws + L.seg_l) : nullptr;
   a.seg_end = split ? (uint32_t*)(ws + L.seg_end) : nullptr;
-  a.max_extra = split ? split_grid(L.seg_max_extra) : 0;
-  a.max_slots = split ? split_grid(L.seg_slots) : 0;
+  a.max_extra = split ? split_grid(L.seg_max_extra, L.seg_max_split) : 0;
+  a.max_slots = split ? split_grid(L.seg_slots, 2 * L.seg_max_split) : 0;
   if (split) return fwd_split<TW, TH>(a, L, ws, st);
   const bool persistent = (cfg.flags & 8) != 0;
   return count ? fwd_launch<TW, TH, true>(a, L, persistent, st) : fwd_launch<TW, TH, false>(a, L, persistent, st);
@@ -1304,7 +1326,7 @@ cudaError_t bwd_t(const Layout& L, const CfgDev& cfg, char* ws, const float* dL,
   a.tile_split = split ? (const uint32_t*)(ws + L.tile_slot) : nullptr;
   a.ext_owner = split ? (const uint32_t*)(ws + L.ext_owner) : nullptr;
   a.seg_c = split ? (const float4*)(ws + L.seg_c) : nullptr;
-  a.max_extra = split ? split_grid(L.seg_max_extra) : 0;
+  a.max_extra = split ? split_grid(L.seg_max_extra, L.seg_max_split) : 0;
   if (split) {
     launch_dependent(render_bwd_kernel<TW, TH, true>, dim3((a.max_extra + L.NT) * (TW * TH / 64)), dim3(32), 0,
                      st, a);

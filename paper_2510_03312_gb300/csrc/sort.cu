@@ -822,29 +822,24 @@ __global__ void __launch_bounds__(kMgT, 2) tile_merge_kernel(const uint2* __rest
     const uint32_t it = s_it;
     if (it >= n_long) break;
     const uint2 item = items[it];
-    if (item.y != 0 && !join) continue;  // uniform over the block
+    if (item.y != 0 && !join) continue;  // uniform over the block, as all that follows
     const uint32_t s = tstart[item.x], L = tstart[item.x + 1] - s;
-    if (join && L > kMergeSeg) {  // one segment; tile_join_kernel does the rest
-      if (item.y % (kMergeSeg / kSortChunk) != 0) continue;
-      const uint32_t s0 = item.y * kSortChunk, n = min(kMergeSeg, L - s0);
-      merge_segment(chunk64 + s + s0, n, s_seg);
-      for (uint32_t i = threadIdx.x; i < n; i += kMgT) chunk64[s + s0 + i] = s_seg[i];
-      __syncthreads();  // the segment buffer is free for the block's next item
-      continue;
-    }
-    if (item.y != 0) continue;
-    if (L <= kMergeSeg) {
-      merge_segment(chunk64 + s, L, s_seg);
-      for (uint32_t i = threadIdx.x; i < L; i += kMgT) out[s + i] = (uint32_t)s_seg[i];
-      __syncthreads();  // the segment buffer is free for the block's next list
-      continue;
-    }
-    for (uint32_t s0 = 0; s0 < L; s0 += kMergeSeg) {
+    // the list's segments; with join, of a list of several, this item's own
+    // (tile_join_kernel does the rest)
+    const bool part = join && L > kMergeSeg;
+    if (part ? item.y % (kMergeSeg / kSortChunk) != 0 : item.y != 0) continue;
+    const uint32_t first = part ? item.y * kSortChunk : 0u, end = part ? first + 1 : L;
+    for (uint32_t s0 = first; s0 < end; s0 += kMergeSeg) {
       const uint32_t n = min(kMergeSeg, L - s0);
       merge_segment(chunk64 + s + s0, n, s_seg);
-      for (uint32_t i = threadIdx.x; i < n; i += kMgT) chunk64[s + s0 + i] = s_seg[i];
-      __syncthreads();
+      if (L <= kMergeSeg) {
+        for (uint32_t i = threadIdx.x; i < n; i += kMgT) out[s + i] = (uint32_t)s_seg[i];
+      } else {
+        for (uint32_t i = threadIdx.x; i < n; i += kMgT) chunk64[s + s0 + i] = s_seg[i];
+      }
+      __syncthreads();  // the segment buffer is free again
     }
+    if (part || L <= kMergeSeg) continue;
     unsigned long long* src = chunk64 + s;
     unsigned long long* dst = tmp64 + s;
     const uint32_t share = (L + kMgT - 1) / kMgT;
