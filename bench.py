@@ -208,13 +208,16 @@ def kernels_per_step(r):
     V, S = len(r.views), len(r.scenes)
     NT = sum(((v.width + r.cfg.tile_w - 1) // r.cfg.tile_w) * ((v.height + r.cfg.tile_h - 1) // r.cfg.tile_h)
              for v in r.views)
-    upload = (V + 15) // 16
+    # one view goes along with its scene's preprocess launch
+    upload = 0 if V == 1 and r.scenes[r.views[0].scene_id].P > 0 else (V + 15) // 16
     pre = upload + S
-    # the count, the scan (two kernels, three over more than 2048 x 1024
-    # tiles; the second also makes the tile order), the scatter, the
-    # per-tile sort and the merge of long lists
+    # the count, the scan (one kernel up to 1024 tiles, else two, three over
+    # more than 2048 x 1024 tiles; the last also makes the tile order), the
+    # scatter, the per-tile sort and the merge of long lists, which makes the
+    # tile descriptors (by themselves where there are no records)
     R = sum(r.scenes[v.scene_id].P for v in r.views)
-    sort = 0 if R == 0 else (1 + 2 + (1 if (NT + 1023) // 1024 > 2048 else 0) + 3)
+    scan = 1 if NT <= 1024 else (3 if (NT + 1023) // 1024 > 2048 else 2)
+    sort = 1 if R == 0 else 1 + scan + 3
     # forward blend; zeroing of the visible records' gradient sums, backward
     # blend; parameter backward per scene
     return pre + sort + 1 + 2 + S
