@@ -895,10 +895,13 @@ __device__ __forceinline__ int writer_of(int lane) {
 //   v7..9 = sum alpha T dL/dC.
 // With dr = -beta q:  d mu' = 2 beta [[a, b], [b, c]] (v0, v1),
 // d(a, b, c) = -beta (v2, 2 v3, v4), d log2 o = ln2 v5, d beta = ln2 v6.
-// dL/dalpha = T (c - B) . dL/dC needs the colour behind, B, only as its
-// product with the pixel's dL/dC, one packed value instead of three: six of
-// some 150 instructions per (entry, block) less, by whose issue the kernel is
-// bound (whole cases: 1M-primitive view 1.8%, uneven batch 1.5%).
+//
+// dL/dalpha = T (c - B) . dL/dC, B the colour behind, is formed from the three
+// differences c - B: they are exact where c is near B, and zero where c is B.
+// One recurrence for B . dL/dC (six of some 150 instructions less, the
+// 1M-primitive step 671 us instead of 684) leaves the rounding of the two
+// products there: with colours within 1e-3 of the background, 1.6 to 5.6
+// times the gradients' error against float64.
 //
 // One CTA of one warp per 8x8 block of a tile (two pixels a lane, rows y and
 // y + 4), with no block-wide barrier: warps of a tile finish independently
@@ -907,7 +910,7 @@ __device__ __forceinline__ int writer_of(int lane) {
 // stages one record, the batch is culled to the entries whose support meets
 // the block, those are processed, and each record the block used is flushed
 // by its lane with one vector atomic add per (record, block).  The pair
-// evaluation and the per-pixel recurrences (T, the colour behind's product) run in
+// evaluation and the per-pixel recurrences (T, the colour behind) run in
 // packed pairs over the lane's two pixels; the two share dx, so a lane's
 // sums of q dx, q dx^2 and q dx dy take dx out of the sum.
 struct BwdSmem {
@@ -960,6 +963,9 @@ __device__ __forceinline__ void bwd_block(const BwdArgs& A, const Tile& v, int w
   const float2 fx = make_float2((float)lx + 0.5f, (float)lx + 0.5f);
   const float2 fy = make_float2((float)ly + 0.5f, (float)(ly + 4) + 0.5f);
   float2 T = make_float2(1.0f, 1.0f), G0 = make_float2(0.0f, 0.0f), G1 = G0, G2 = G0;
+  // colour behind the current record, normalised by the transmittance after it
+  float2 B0 = make_float2(cfg.bg[0], cfg.bg[0]), B1 = make_float2(cfg.bg[1], cfg.bg[1]),
+         B2 = make_float2(cfg.bg[2], cfg.bg[2]);
   uint32_t last0 = 0, last1 = 0;
   {
     const size_t plane = (size_t)v.W * v.H;
@@ -982,25 +988,22 @@ __device__ __forceinline__ void bwd_block(const BwdArgs& A, const Tile& v, int w
       last1 = A.lastc[v.pix + pix];
     }
   }
-  // -B . dL/dC, B the colour behind the current record normalised by the
-  // transmittance after it: the recurrence needs B only so
-  auto behind = [](float b0, float b1, float b2, float g0, float g1, float g2) {
-    return -fmaf(b0, g0, fmaf(b1, g1, b2 * g2));
-  };
-  float2 N = make_float2(behind(cfg.bg[0], cfg.bg[1], cfg.bg[2], G0.x, G1.x, G2.x),
-                         behind(cfg.bg[0], cfg.bg[1], cfg.bg[2], G0.y, G1.y, G2.y));
   if constexpr (SPLIT) {
     // the segment's end: T and the normalised colour behind it, for the pixels
     // whose walk reaches the segment (the others use no entry of it)
     if (slot && last0 > wbeg) {
       const float4 s0 = slot[ly * TW + lx];
       T.x = s0.w;
-      N.x = behind(s0.x, s0.y, s0.z, G0.x, G1.x, G2.x);
+      B0.x = s0.x;
+      B1.x = s0.y;
+      B2.x = s0.z;
     }
     if (slot && last1 > wbeg) {
       const float4 s1 = slot[(ly + 4) * TW + lx];
       T.y = s1.w;
-      N.y = behind(s1.x, s1.y, s1.z, G0.y, G1.y, G2.y);
+      B0.y = s1.x;
+      B1.y = s1.y;
+      B2.y = s1.z;
     }
   }
   const float ox = (float)v.x0, oy = (float)v.y0;
@@ -1028,7 +1031,7 @@ __device__ __forceinline__ void bwd_block(const BwdArgs& A, const Tile& v, int w
     if (wlast <= wbeg) return;
   }
   if (wlast == 0) return;
-  const float2 one = make_float2(1.0f, 1.0f);
+  const float2 one = make_float2(1.0f, 1.0f), neg1 = make_float2(-1.0f, -1.0f);
   const int wslot = writer_of(lane);
   const int wfirst = SPLIT ? (int)wbeg : 0;
   for (int hi = (int)wlast; hi > wfirst; hi -= WB) {
@@ -1055,23 +1058,26 @@ __device__ __forceinline__ void bwd_block(const BwdArgs& A, const Tile& v, int w
       const unsigned hits = __ballot_sync(kFull, use0 || use1);
       if (hits == 0) continue;  // no pixel of the block: T and B stay
       touched |= 1u << j;
-      // branch-free: a pair the forward skipped contributes zero and leaves T, N.
-      // The pair's sums carry -alpha's sign; the flush takes it back.
-      const float2 na = make_float2(use0 ? -e.alpha.x : 0.0f, use1 ? -e.alpha.y : 0.0f);
-      const float2 oma = add2(one, na);
+      // branch-free: a pair the forward skipped contributes zero and leaves T, B
+      const float2 a = make_float2(use0 ? e.alpha.x : 0.0f, use1 ? e.alpha.y : 0.0f);
+      const float2 oma = fma2(a, neg1, one);
       T = mul2(T, make_float2(rcp_approx(oma.x), rcp_approx(oma.y)));  // transmittance before this record
-      const float2 w = mul2(na, T);
+      const float2 w = mul2(a, T);
       float gv[10];
       {
-        const float2 eg = fma2(hi2(D), G0, fma2(lo2(E), G1, fma2(hi2(E), G2, N)));  // (c - B) . dL/dC
-        N = fma2(na, eg, N);
+        const float2 c0 = hi2(D), c1 = lo2(E), c2 = hi2(E);
+        const float2 e0 = fma2(B0, neg1, c0), e1 = fma2(B1, neg1, c1), e2 = fma2(B2, neg1, c2);
+        const float2 dal = mul2(T, fma2(e0, G0, fma2(e1, G1, mul2(e2, G2))));
+        B0 = fma2(a, e0, B0);
+        B1 = fma2(a, e1, B1);
+        B2 = fma2(a, e2, B2);
         const float2 wg0 = mul2(w, G0), wg1 = mul2(w, G1), wg2 = mul2(w, G2);
         gv[7] = wg0.x + wg0.y;
         gv[8] = wg1.x + wg1.y;
         gv[9] = wg2.x + wg2.y;
-        float2 ga = mul2(w, eg);
-        ga.x = e.alpha.x < cfg.amax ? ga.x : 0.0f;
-        ga.y = e.alpha.y < cfg.amax ? ga.y : 0.0f;
+        float2 ga = mul2(dal, a);
+        ga.x = a.x < cfg.amax ? ga.x : 0.0f;
+        ga.y = a.y < cfg.amax ? ga.y : 0.0f;
         // q = ga / (1 - r): ga = 0 unless composited, and 1 - r > 0
         const float2 qq = mul2(ga, make_float2(rcp_approx(e.om.x), rcp_approx(e.om.y)));
         const float2 u1 = mul2(qq, e.dy);
@@ -1101,11 +1107,11 @@ __device__ __forceinline__ void bwd_block(const BwdArgs& A, const Tile& v, int w
       const float a = sm.st[lane].Bc.x, b = 0.5f * sm.st[lane].Bc.z, c = sm.st[lane].Cc.x, beta = sm.st[lane].Cc.z;
       const float v0 = sm.acc[0][lane], v1 = sm.acc[1][lane];
       float4* dst = A.g2d + 3 * (size_t)sm.rec[lane];
-      atomicAdd(dst, make_float4(-2.0f * beta * (a * v0 + b * v1), -2.0f * beta * (b * v0 + c * v1),
-                                 beta * sm.acc[2][lane], 2.0f * beta * sm.acc[3][lane]));
-      atomicAdd(dst + 1, make_float4(beta * sm.acc[4][lane], -kLn2f * sm.acc[5][lane], -kLn2f * sm.acc[6][lane],
-                                     -sm.acc[7][lane]));
-      atomicAdd((float2*)(dst + 2), make_float2(-sm.acc[8][lane], -sm.acc[9][lane]));
+      atomicAdd(dst, make_float4(2.0f * beta * (a * v0 + b * v1), 2.0f * beta * (b * v0 + c * v1),
+                                 -beta * sm.acc[2][lane], -2.0f * beta * sm.acc[3][lane]));
+      atomicAdd(dst + 1, make_float4(-beta * sm.acc[4][lane], kLn2f * sm.acc[5][lane], kLn2f * sm.acc[6][lane],
+                                     sm.acc[7][lane]));
+      atomicAdd((float2*)(dst + 2), make_float2(sm.acc[8][lane], sm.acc[9][lane]));
     }
     __syncwarp();
   }

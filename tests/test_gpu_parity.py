@@ -452,3 +452,24 @@ def test_empty_scenes():
     g = r.backward(dl.view_as(both["image_flat"]))
     torch.cuda.synchronize()
     assert g[0].numel() == 0 and torch.isfinite(g[1]).all() and float(g[1].abs().max()) > 0
+
+
+@pytest.mark.parametrize("N,form,tile", [(3, "grid", (16, 16)), (3, "persistent", (8, 8)), (3, "split", (16, 16)),
+                                         (6, "grid", (16, 32))])
+def test_colours_of_the_background_leave_no_gradient(N, form, tile):
+    """Where every primitive has the background's colour, no pixel changes
+    with the geometry or the opacities: the colour behind a record equals the
+    record's exactly, so their gradients are zero to the last bit, whatever
+    dL/dimage is; the colours' own gradients are not."""
+    scenes, views, _ = _multi(N, 6000, 2, 150, 110, 23)
+    bg = (0.83, 0.61, 0.37)
+    scenes[0].plane("rgb")[:] = np.array(bg, np.float32)[:, None]
+    cfg = S.RasterConfig(tile_w=tile[0], tile_h=tile[1], bg=bg, persistent=form == "persistent",
+                         split_lists=form == "split")
+    gpu = gpu_forward(scenes, views, cfg)
+    r = gpu["rast"]
+    dL = torch.randn(r.image.numel(), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    g = r.backward(dL)[0].cpu().numpy()
+    n_rgb = 3
+    assert np.abs(g[-n_rgb:]).max() > 0.0
+    assert np.abs(g[:-n_rgb]).max() == 0.0
