@@ -4,11 +4,14 @@
 // Compiled with --fmad=false -prec-div=true -prec-sqrt=true -ftz=false so
 // that the float32 rule set of spec32.cuh holds (see prim_forward.cuh).
 //
-// One thread per primitive of one scene; the thread builds the view-
-// independent part once (Sigma blocks, Cholesky of Sigma_q, Sigma_q^{-1}
-// Sigma_qx, beta) and then loops over the scene's views, so each primitive's
-// parameters are read from HBM once per batch of views.  Parameter planes
-// are structure-of-arrays: a warp reads 32 consecutive floats per plane.
+// One launch per scene.  A primitive's view-independent part (Sigma blocks,
+// Cholesky of Sigma_q, Sigma_q^{-1} Sigma_qx, beta) is built once for all the
+// scene's views, so its parameters are read from HBM once per batch of views.
+// Three forms (launch_preprocess): a thread per primitive that loops over the
+// views (N = 3, and small scenes of one view); for one view of a larger scene
+// with query dimensions, a cheap test before anything else; for several, that
+// test per view and a queue of the records that pass.  Parameter planes are
+// structure-of-arrays: a warp reads 32 consecutive floats per plane.
 #include <atomic>
 
 #include "kernels.cuh"
@@ -253,6 +256,15 @@ __device__ __forceinline__ bool certain_cull_one(const PrimIn<C>& in, float belo
 // 17.6 us so; 200K N=6, 7% drawn: 22 -> 14.6.  Held to 64 registers, so that
 // these grids are one wave (at 80 registers 23 and 14.3 us, at 128 23 and 21).
 constexpr int kOneThreads = 256, kOnePrims = 512;
+// Below kOneMin primitives preprocess_kernel takes the scene, in CTAs of
+// kFewThreads: its grid then fills the GPU where that of kOnePrims a CTA does
+// not, and there is no second read.  Forward of one 640x360 view, that / this
+// form, us: 20K N=7 31 / 35 where the query culls almost all and 50 / 61 where
+// it culls none; 80K 37 / 38 and 104 / 116; 100K 41 / 39 and 125 / 134; 300K
+// 62 / 50 and 201 / 207.  From the line on the test pays where the query culls
+// and costs at most 7% where it does not.
+constexpr int64_t kOneMin = 100000;
+constexpr int kFewThreads = 64;
 template <int C>
 __global__ void __launch_bounds__(kOneThreads, 4) preprocess_one_view_kernel(
     SceneDev sc, ViewList vl, const ViewDev* __restrict__ views, CfgDev cfg, float4* __restrict__ rec4,
@@ -498,19 +510,23 @@ cudaError_t launch_preprocess(const SceneDev& sc, const ViewList& vl, const View
                               const Layout& L, char* ws, uint32_t* act_list, uint32_t* act_count, uint32_t* zero,
                               uint32_t nzero, const OneView& one, cudaStream_t st) {
   if (sc.P == 0 || vl.n == 0) return cudaSuccess;
-  if (sc.N > 3) {
-    const cudaError_t e = prepare_queued();
-    if (e != cudaSuccess) return e;
-  }
-  const int threads = sc.N > 3 ? kQThreads : 256;
-  const unsigned blocks = (unsigned)((sc.P + threads - 1) / threads);
-  const size_t smem = sizeof(ViewDev) * vl.n;
   float4* rec4 = (float4*)(ws + L.rec4);
   uint32_t* key = (uint32_t*)(ws + L.key);
   uint32_t* tiles = (uint32_t*)(ws + L.tiles);
   uint2* rect = (uint2*)(ws + L.rect);
   uint32_t* vis = (uint32_t*)(ws + L.vis_mask);
+  const size_t smem = sizeof(ViewDev) * vl.n;
   if (sc.N > 3 && vl.n == 1) {
+    if (sc.P < kOneMin) {
+      const dim3 grid((unsigned)((sc.P + kFewThreads - 1) / kFewThreads)), block(kFewThreads);
+      switch (sc.N) {
+        case 4: launch_dependent(preprocess_kernel<1>, grid, block, smem, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, act_list, act_count, zero, nzero, one); break;
+        case 6: launch_dependent(preprocess_kernel<3>, grid, block, smem, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, act_list, act_count, zero, nzero, one); break;
+        case 7: launch_dependent(preprocess_kernel<4>, grid, block, smem, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, act_list, act_count, zero, nzero, one); break;
+        default: return cudaErrorInvalidValue;
+      }
+      return cudaGetLastError();
+    }
     const dim3 grid((unsigned)((sc.P + kOnePrims - 1) / kOnePrims)), block(kOneThreads);
     switch (sc.N) {
       case 4: launch_dependent(preprocess_one_view_kernel<1>, grid, block, 0, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, zero, nzero, one); break;
@@ -520,6 +536,12 @@ cudaError_t launch_preprocess(const SceneDev& sc, const ViewList& vl, const View
     }
     return cudaGetLastError();
   }
+  if (sc.N > 3) {
+    const cudaError_t e = prepare_queued();
+    if (e != cudaSuccess) return e;
+  }
+  const int threads = sc.N > 3 ? kQThreads : 256;
+  const unsigned blocks = (unsigned)((sc.P + threads - 1) / threads);
   switch (sc.N) {
     case 3: launch_dependent(preprocess_kernel<0>, dim3(blocks), dim3(threads), smem, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, act_list, act_count, zero, nzero, one); break;
     case 4: launch_dependent(preprocess_queued_kernel<1>, dim3(blocks), dim3(threads), smem, st, sc, vl, views, cfg, rec4, key, tiles, rect, vis, act_list, act_count, zero, nzero); break;

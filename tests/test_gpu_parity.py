@@ -473,3 +473,12 @@ def test_colours_of_the_background_leave_no_gradient(N, form, tile):
     n_rgb = 3
     assert np.abs(g[-n_rgb:]).max() > 0.0
     assert np.abs(g[:-n_rgb]).max() == 0.0
+
+
+@pytest.mark.parametrize("N", [4, 6, 7])
+@pytest.mark.parametrize("P", [63, 64, 65, 99_999, 100_000, 100_033])
+def test_query_cull_at_extremes_of_one_view(N, P):
+    """As above for one view, on both sides of the size from which the cheap
+    test comes before the view-independent stage, and at a CTA's edges of the
+    form for fewer primitives."""
+    test_query_cull_at_extremes(N, P, 1)
