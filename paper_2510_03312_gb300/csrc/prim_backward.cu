@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(128, C == 0 ? 7 : 1) prim_backward_kernel(Scen
 }
 
 
-// Scenes with query dimensions and one view: one CTA per kPbPrims consecutive
+// Scenes with query dimensions and one view: one CTA per `prims` consecutive
 // primitives.  It lists those the view draws (their visibility bits) in shared
 // memory and gives each thread listed ones, whose parameters lie close
 // together; then it writes zero gradients for the others (unless
@@ -90,18 +90,39 @@ __global__ void __launch_bounds__(128, C == 0 ? 7 : 1) prim_backward_kernel(Scen
 // primitives: 40 us; 17 us so).  Scenes with several views draw most primitives
 // in some view: there the list of the whole scene (prim_backward_listed_kernel)
 // balances better (16 views of 500K N=6 primitives: 11 + 98 us, this form 144).
+// How many are drawn is not known at the launch.  Where few are, a CTA's time
+// is one round's latency and long ranges win; where nearly all are, a long
+// range takes several rounds, and a grid that ends in a nearly empty wave waits
+// for all of them.  So the range is the longest (128, 256, 384 or 512) whose
+// rounds, with every primitive drawn, number at most 5/4 of the fewest that any
+// length gives.  Whole step of one 640x360 view by ranges of 128 / 256 / 512,
+// us (a thread per primitive before): N=7 30K primitives, 1% drawn 48 / 48 / 48
+// (56), 86% drawn 107 / 113 / 124 (116); 60K 57 / 52 / 53 (65) and 176 / 176 /
+// 187 (185); 160K 75 / 67 / 65 (97) and 343 / 349 / 366 (343); 300K 106 / 93 /
+// 81 (142) and 416 / 413 / 414 (423); N=6 60K, 6% drawn 56 / 56 / 56 (69), 92%
+// drawn 181 / 185 / 198 (193); 200K 91 / 87 / 83 (120) and 304 / 310 / 308
+// (329).
 constexpr int kPbThreads = 128;
 constexpr int kPbPrims = 512, kPbWords = kPbPrims / 32;
+inline int pb_prims(int N, int64_t P) {
+  const int64_t slots = 152 * (N == 7 ? 2 : 4);  // 205 registers a thread, 128
+  auto rounds = [&](int64_t r) { return r * (((P + r * kPbThreads - 1) / (r * kPbThreads) + slots - 1) / slots); };
+  int64_t least = rounds(1);
+  int r = kPbPrims / kPbThreads;
+  for (int i = 2; i <= r; ++i) least = rounds(i) < least ? rounds(i) : least;
+  while (r > 1 && 4 * rounds(r) > 5 * least) --r;
+  return r * kPbThreads;
+}
 template <int C>
 __global__ void __launch_bounds__(kPbThreads, C == 3 ? 4 : 1) prim_backward_drawn_kernel(
     SceneDev sc, SceneGradDev gr, ViewList vl, const ViewDev* __restrict__ views, CfgDev cfg,
-    const uint32_t* __restrict__ vis_mask, const float4* __restrict__ g2d) {
+    const uint32_t* __restrict__ vis_mask, const float4* __restrict__ g2d, int prims) {
   wait_prior_grid();
   __shared__ ViewDev s_view;
   __shared__ uint32_t s_any[kPbWords], s_first[kPbWords + 1];
   __shared__ uint16_t s_list[kPbPrims];
-  const int64_t P = sc.P, p0 = (int64_t)blockIdx.x * kPbPrims;
-  const uint32_t w0 = (uint32_t)(p0 >> 5), n_words = (uint32_t)min((int64_t)kPbWords, (P + 31) / 32 - (int64_t)w0);
+  const int64_t P = sc.P, p0 = (int64_t)blockIdx.x * prims;
+  const uint32_t w0 = (uint32_t)(p0 >> 5), n_words = (uint32_t)min((int64_t)(prims / 32), (P + 31) / 32 - (int64_t)w0);
   const ViewDev& vd = views[vl.idx[0]];
   if (threadIdx.x < kPbWords) s_any[threadIdx.x] = threadIdx.x < n_words ? vis_mask[vd.mask_off + w0 + threadIdx.x] : 0u;
   if (threadIdx.x == 0) s_view = vd;
@@ -120,7 +141,7 @@ __global__ void __launch_bounds__(kPbThreads, C == 3 ? 4 : 1) prim_backward_draw
   __syncthreads();
   const bool add = (cfg.flags & 4) != 0;  // add to the caller's running sum (UBS_FLAG_ACCUMULATE_GRADS)
   const int nr = sc.rot_mode == 0 ? 4 : 3;
-  for (int i = threadIdx.x; i < kPbPrims; i += kPbThreads) {
+  for (int i = threadIdx.x; i < prims; i += kPbThreads) {
     const uint32_t any = s_any[i >> 5], bit = 1u << (i & 31);
     if (any & bit) s_list[s_first[i >> 5] + __popc(any & (bit - 1u))] = (uint16_t)i;
   }
@@ -156,7 +177,7 @@ __global__ void __launch_bounds__(kPbThreads, C == 3 ? 4 : 1) prim_backward_draw
   }
   if (add) return;
 #pragma unroll 1
-  for (int i = threadIdx.x; i < kPbPrims; i += kPbThreads) {
+  for (int i = threadIdx.x; i < prims; i += kPbThreads) {
     const int64_t p = p0 + i;
     if (p >= P || ((s_any[i >> 5] >> (i & 31)) & 1u)) continue;
     for (int j = 0; j < 3; ++j) gr.mean_x[j * P + p] = 0.0f;
@@ -269,12 +290,13 @@ cudaError_t launch_prim_backward(const SceneDev& sc, const SceneGradDev& g, cons
   const float4* g2d = (const float4*)(ws + L.g2d);
   cudaError_t e = cudaSuccess;
   if (vl.n == 1 && sc.N > 3) {  // the drawn primitives of each CTA's range
-    const dim3 grid((unsigned)((sc.P + kPbPrims - 1) / kPbPrims));
+    const int prims = pb_prims(sc.N, sc.P);
+    const dim3 grid((unsigned)((sc.P + prims - 1) / prims));
     const uint32_t* vis = (const uint32_t*)(ws + L.vis_mask);
     switch (sc.N) {
-      case 4: e = launch_dependent(prim_backward_drawn_kernel<1>, grid, dim3(kPbThreads), 0, st, sc, g, vl, views, cfg, vis, g2d); break;
-      case 6: e = launch_dependent(prim_backward_drawn_kernel<3>, grid, dim3(kPbThreads), 0, st, sc, g, vl, views, cfg, vis, g2d); break;
-      case 7: e = launch_dependent(prim_backward_drawn_kernel<4>, grid, dim3(kPbThreads), 0, st, sc, g, vl, views, cfg, vis, g2d); break;
+      case 4: e = launch_dependent(prim_backward_drawn_kernel<1>, grid, dim3(kPbThreads), 0, st, sc, g, vl, views, cfg, vis, g2d, prims); break;
+      case 6: e = launch_dependent(prim_backward_drawn_kernel<3>, grid, dim3(kPbThreads), 0, st, sc, g, vl, views, cfg, vis, g2d, prims); break;
+      case 7: e = launch_dependent(prim_backward_drawn_kernel<4>, grid, dim3(kPbThreads), 0, st, sc, g, vl, views, cfg, vis, g2d, prims); break;
       default: return cudaErrorInvalidValue;
     }
     return e != cudaSuccess ? e : cudaGetLastError();

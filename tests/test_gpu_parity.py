@@ -482,3 +482,43 @@ def test_query_cull_at_extremes_of_one_view(N, P):
     test comes before the view-independent stage, and at a CTA's edges of the
     form for fewer primitives."""
     test_query_cull_at_extremes(N, P, 1)
+
+
+@pytest.mark.parametrize("N,P", [(4, 65), (6, 80_129), (6, 160_001), (6, 300_000), (7, 129), (7, 40_193), (7, 130_048),
+                                 (7, 160_000)])
+@pytest.mark.parametrize("broad", [False, True])
+def test_one_view_parameter_gradients_match_several(N, P, broad):
+    """Parameter gradients of one view, at sizes that take ranges of 128, 256,
+    384 and 512 primitives with full and ragged last ones, against the same
+    view beside a second one that gets no gradient (scenes with several views
+    take the scene's own list): within the float atomics' rounding, with the
+    same primitives untouched, where the query culls most records and where it
+    culls few; written and accumulated."""
+    rng = np.random.default_rng(P + N)
+    sc = S.make_scene(P, N, P, means="clusters", extent=2.0, n_clusters=8, rng=rng)
+    if broad:
+        for name in ("L_qx", "L_q"):
+            sc.plane(name)[:] *= 8.0
+        sc.plane("b")[1:] -= 2.0
+    views = S.sphere_views(rng, 2, 5.0, 96, 80, hemisphere=True, times=[0.3, 0.6])
+    got = []
+    for vs in (views[:1], views):
+        ds = raster.DeviceScene.from_scene(sc, device="cuda")
+        r = raster.Rasterizer([ds], vs, S.RasterConfig(), device="cuda")
+        r.forward(check=True)
+        n = 3 * views[0].width * views[0].height
+        dL = torch.zeros(r.image.numel(), device="cuda")
+        dL[:n] = torch.sin(torch.arange(n, device="cuda")) / n
+        got.append(r.backward(dL)[0].clone())
+        drawn = int(r.status().visible_records)
+        acc = raster.Rasterizer([ds], vs, S.RasterConfig(), device="cuda", accumulate=True,
+                                grads=[torch.ones_like(got[-1])])
+        acc.forward(check=True)
+        more = acc.backward(dL)[0]
+        # 1 + g in float32: one rounding of a number near 1, and the atomics'
+        assert (more - 1.0 - got[-1]).abs().max() <= 2.0 ** -23 * (1.0 + got[-1].abs().max()) + 1e-5 * got[-1].abs().max()
+    one, two = got
+    assert drawn > 0 and (P < 1000 or one.abs().amax(1).min() > 0)
+    assert torch.equal((one != 0).any(0), (two != 0).any(0))
+    worst = ((one - two).abs().amax(1) / two.abs().amax(1).clamp(min=1e-30)).max()
+    assert worst <= 1e-5, float(worst)
