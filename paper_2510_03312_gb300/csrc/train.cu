@@ -21,7 +21,7 @@
 // for four neighbouring columns, the warp exchanges those sums, and a row's
 // sums enter the column's ten unfinished column sums, held in registers (sum i
 // becomes sum i + 1 plus its tap: nothing is shifted or staged).  The strips'
-// height is chosen so that all CTAs are resident at once.
+// height is chosen so that all CTAs are resident at once, up to 96 rows.
 //   ssim_fwd_kernel   the five window statistics, S, the three partials (to
 //                     the workspace) and per-block sums of S and |x - y|
 //   ssim_bwd_kernel   the three partials convolved back, combined with the
@@ -549,26 +549,39 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-bool loss_views(int32_t n, const int32_t* w, const int32_t* h, LossParams* P, size_t* ws) {
+int sm_count() {
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+// Sizes and, with P, the blocks of the two kernels on a device of `sms` SMs.
+bool loss_blocks(int32_t n, const int32_t* w, const int32_t* h, int sms, LossParams* P, size_t* ws) {
   if (n < 1 || n > kLossMaxViews || !w || !h) return false;
-  uint64_t pix = 0, sums = 0, cols = 0;
+  uint64_t pix = 0, sums = 0;
   for (int i = 0; i < n; ++i) {
     if (w[i] < 1 || h[i] < 1 || w[i] > 65535 || h[i] > 65535) return false;
     pix += (uint64_t)w[i] * h[i];
     sums += 3ull * ((w[i] + kSumTile - 1) / kSumTile) * ((h[i] + kSumTile - 1) / kSumTile);
-    cols += 3ull * ((w[i] + kLT - 1) / kLT) * h[i];
     if (pix > 0x7fffffffull / 3 || sums > 0x7fffffffull) return false;
   }
   *ws = align256(3 * 3 * pix * sizeof(float)) + align256(sums * sizeof(float2));
   if (!P) return true;
-  // The strips' height: as many strips as CTAs fit on the GPU, a multiple of
-  // the step, between kMinRows (each strip also walks 2 kRad halo rows: 16 and
-  // 24 rows took 150 and 148 us for a training step at 800 x 600, 32 took 147)
-  // and kMaxRows; as kMinRows >= kSumTile there is a block sum for each
+  // The strips' height: a multiple of the step, between kMinRows (each strip
+  // also walks 2 kRad halo rows: 16 and 24 rows took 150 and 148 us for a
+  // training step at 800 x 600, 32 took 147) and kMaxRows, and in between the
+  // least for which all CTAs, the backward's reducing one too, are resident at
+  // once (1920 x 1080 with five strips too many 112 us, so 97); as kMinRows >=
+  // kSumTile there is a block sum for each
   static_assert(kMinRows >= kSumTile && kMinRows % kLR == 0 && kLT >= kSumTile, "a block sum per strip");
-  const uint64_t ctas = 152ull * kLossCtas;
-  uint64_t rows = ((cols + ctas - 1) / ctas + kLR - 1) / kLR * kLR;
-  rows = rows < kMinRows ? kMinRows : (rows > kMaxRows ? kMaxRows : rows);
+  uint64_t rows = kMinRows;
+  auto blocks = [&](uint64_t r) {
+    uint64_t k = 1;
+    for (int i = 0; i < n; ++i) k += 3ull * ((w[i] + kLT - 1) / kLT) * ((h[i] + r - 1) / r);
+    return k;
+  };
+  while (rows < kMaxRows && blocks(rows) > (uint64_t)sms * kLossCtas) rows += kLR;
   uint64_t blk = 0, at = 0;
   for (int i = 0; i < n; ++i) {
     LossView& v = P->v[i];
@@ -595,22 +608,23 @@ using namespace ubs;
 
 extern "C" size_t ubs_loss_workspace_size(int32_t n_views, const int32_t* widths, const int32_t* heights) {
   size_t ws = 0;
-  return loss_views(n_views, widths, heights, nullptr, &ws) ? ws : 0;
+  return loss_blocks(n_views, widths, heights, 0, nullptr, &ws) ? ws : 0;
 }
 
 extern "C" ubs_status ubs_image_loss(int32_t n_views, const int32_t* widths, const int32_t* heights,
                                      const float* image, const float* target, float lambda_ssim, float* dL_dimage,
                                      float* loss, void* workspace, size_t workspace_bytes, cudaStream_t stream) {
   ubs::TraceRange trace_("ubs_image_loss");
-  LossParams p;
-  memset(&p, 0, sizeof(p));
   size_t need = 0;
-  if (!loss_views(n_views, widths, heights, &p, &need)) return UBS_ERR_INVALID_ARG;
+  if (!loss_blocks(n_views, widths, heights, 0, nullptr, &need)) return UBS_ERR_INVALID_ARG;
   if (!image || !target || !dL_dimage || !loss || !workspace) return UBS_ERR_INVALID_ARG;
   if (!(lambda_ssim >= 0.0f && lambda_ssim <= 1.0f)) return UBS_ERR_INVALID_ARG;
   if (((uintptr_t)workspace & 255u) != 0) return UBS_ERR_ALIGNMENT;
   if (((uintptr_t)image | (uintptr_t)target | (uintptr_t)dL_dimage | (uintptr_t)loss) & 3u) return UBS_ERR_ALIGNMENT;
   if (workspace_bytes < need) return UBS_ERR_WORKSPACE;
+  LossParams p;
+  memset(&p, 0, sizeof(p));
+  loss_blocks(n_views, widths, heights, sm_count(), &p, &need);
   // the 1-D window: exp(-(i - 5)^2 / (2 * 1.5^2)), normalised to sum 1
   double g[kWin], s = 0.0;
   for (int i = 0; i < kWin; ++i) {
@@ -668,9 +682,7 @@ extern "C" ubs_status ubs_adam_step(int32_t K, int64_t P, const ubs_adam_plane* 
   // the words' arrays; the noise may lie anywhere
   const bool vec = (((uintptr_t)raw | (uintptr_t)act_out | (uintptr_t)grad | (uintptr_t)m | (uintptr_t)v) & 15u) == 0;
   const int64_t units = vec ? (int64_t)K * P / 4 + 1 : (int64_t)K * P;
-  int dev = 0, sms = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = sm_count();
   const int64_t want = (units + 255) / 256;
   const unsigned grid = (unsigned)(want < (int64_t)sms * 8 ? want : (int64_t)sms * 8);
   cudaError_t e = vec ? launch_dependent(adam_kernel<true>, dim3(grid), dim3(256), 0, stream, A, raw, act_out, grad, m,
