@@ -21,7 +21,8 @@
 // for four neighbouring columns, the warp exchanges those sums, and a row's
 // sums enter the column's ten unfinished column sums, held in registers (sum i
 // becomes sum i + 1 plus its tap: nothing is shifted or staged).  The strips'
-// height is chosen so that all CTAs are resident at once, up to 96 rows.
+// height is chosen so that all CTAs are resident at once, up to 96 rows.  Few or
+// narrow images go by 32 x 32 tiles instead (use_tiles).
 //   ssim_fwd_kernel   the five window statistics, S, the three partials (to
 //                     the workspace) and per-block sums of S and |x - y|
 //   ssim_bwd_kernel   the three partials convolved back, combined with the
@@ -58,17 +59,17 @@ constexpr uint64_t kMinRows = 32, kMaxRows = 96;  // height of a strip
 constexpr float kC1 = 0.0001f, kC2 = 0.0009f;  // (0.01)^2, (0.03)^2
 
 struct LossView {
-  int32_t W, H, tiles_x;  // strips across
+  int32_t W, H, tiles_x;  // blocks (strips or tiles) across
   uint32_t pix_off;       // first pixel of the view
-  uint32_t blk_off;       // first strip of the view
-  int32_t tiles;          // strips per channel
+  uint32_t blk_off;       // first block of the view
+  int32_t tiles;          // blocks per channel
 };
 struct LossParams {
   LossView v[kLossMaxViews];
   float2 g2[kRad + 1]; // 1-D window (g_k, g_k), g_k = g_(10 - k), sums to 1
-  int32_t rows;        // output rows of a strip
+  int32_t cols, rows;  // output columns and rows of a block
   int32_t n;           // views
-  uint32_t n_blocks;   // strips
+  uint32_t n_blocks;   // blocks
   float lam;           // lambda_SSIM
   float inv_views;     // 1 / n
   uint64_t plane;      // floats in one partial plane (3 * all pixels)
@@ -100,7 +101,7 @@ __device__ __forceinline__ StripAt strip_at(const LossParams& P, uint32_t block)
   StripAt s;
   s.W = w.W;
   s.H = w.H;
-  s.gx0 = (ti % w.tiles_x) * kLT;
+  s.gx0 = (ti % w.tiles_x) * P.cols;
   s.gy0 = (ti / w.tiles_x) * P.rows;
   s.rows = min(P.rows, w.H - s.gy0);
   s.base = (size_t)w.pix_off * 3 + (size_t)ch * w.W * w.H;
@@ -311,10 +312,11 @@ __global__ void __launch_bounds__(kLT, kLossCtas)
 // The losses from the block sums, by one CTA: a warp per view in turn, its
 // lanes' strided sums in a fixed shuffle tree, then the views in order
 // (deterministic).  s_view: kLossMaxViews floats.
+template <int NT>
 __device__ __forceinline__ void loss_reduce(const LossParams& P, const float2* __restrict__ bsum,
                                             float* __restrict__ loss, float* s_view) {
   const int lane = threadIdx.x & 31;
-  for (int v = threadIdx.x >> 5; v < P.n; v += kLT / 32) {
+  for (int v = threadIdx.x >> 5; v < P.n; v += NT / 32) {
     const LossView& w = P.v[v];
     const uint32_t nb = 3u * (uint32_t)w.tiles;
     float s = 0.0f, l = 0.0f;
@@ -354,7 +356,7 @@ __global__ void __launch_bounds__(kLT, kLossCtas)
   __shared__ __align__(16) float2 xp[kLT / 32][kXPair];  // row sums of both
   __shared__ __align__(16) float xc[kLT / 32][kXOne];
   if (blockIdx.x == 0) {
-    loss_reduce(P, bsum, loss, reinterpret_cast<float*>(sp));
+    loss_reduce<kLT>(P, bsum, loss, reinterpret_cast<float*>(sp));
     return;
   }
   const StripAt s = strip_at(P, blockIdx.x - 1);
@@ -444,6 +446,267 @@ __global__ void __launch_bounds__(kLT, kLossCtas)
       // d(1 - SSIM)/dx = -dSSIM/dx
       at_bytes(dst, o0 + (uint32_t)r * rowb) = w1 * sg - ws * (fm.x + 2.0f * x * fm.y + y * fc);
     }
+  }
+}
+
+// ---------------------------------------------------------------- small images
+//
+// A CTA per 32 x 32 tile, staged whole with its halo, both passes through
+// shared memory: more arithmetic and shared-memory traffic per pixel than a
+// strip, but a single step, and all tiles at once (see loss_blocks).
+constexpr int kTX = 32, kTY = 32;       // output tile
+constexpr int kHY = kTY + 2 * kRad;     // halo rows
+constexpr int kCOff = 8;                // shared-memory column of tile column 0
+constexpr int kSW = kCOff + kTX + 8;    // shared-memory row: tile columns -8 .. 39
+constexpr int kTileThreads = 256;
+constexpr int kTileCtas = 5;            // CTAs per SM
+static_assert(kTX == kSumTile && kTY == kSumTile, "a block sum per tile");
+
+__device__ __forceinline__ float2 tap(const LossParams& P, int k) { return P.g2[k <= kRad ? k : kWin - 1 - k]; }
+
+// Fills the tile with its halo (rows -5 .. 36, columns -8 .. 39 of the tile)
+// in shared memory, zero outside the image, with asynchronous copies: one
+// warp per row, each lane two columns, every copy of the thread in flight
+// before it waits.  copy(r, c, offset, in) issues the copies of one element
+// (offset: of the pixel within its plane set; clamped to the tile's first
+// pixel when !in).
+template <typename Copy>
+__device__ __forceinline__ void load_halo(const StripAt& t, Copy copy) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int gxa = t.gx0 - kCOff + lane, gxb = gxa + 32;
+  const bool ca = gxa >= 0 && gxa < t.W, cb = lane < kSW - 32 && gxb >= 0 && gxb < t.W;
+  constexpr int kRows = (kHY + kTileThreads / 32 - 1) / (kTileThreads / 32);
+#pragma unroll
+  for (int i = 0; i < kRows; ++i) {
+    const int r = warp + i * (kTileThreads / 32);
+    if (r < kHY) {
+      const int gy = t.gy0 - kRad + r;
+      const bool ry = gy >= 0 && gy < t.H;
+      const size_t row = t.base + (size_t)(ry ? gy : t.gy0) * t.W;
+      copy(r, lane, row + (ry && ca ? gxa : t.gx0), ry && ca);
+      if (lane < kSW - 32) copy(r, lane + 32, row + (ry && cb ? gxb : t.gx0), ry && cb);
+    }
+  }
+  cp_async_wait_all();
+}
+
+// Row pass over one halo row r: the 11-tap window sums at output columns c0
+// and c0 + 1 (tile coordinates), from the 16-byte words of shared columns
+// c0 + 2 .. c0 + 15 (tile columns c0 - 6 .. c0 + 7).  F receives each loaded
+// column with, per output o, its tap k (or -1).
+template <typename F>
+__device__ __forceinline__ void row_taps(int c0, F f) {
+#pragma unroll
+  for (int ch = 0; ch < 7; ++ch)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int j = 2 * ch + e;  // tile column c0 - 6 + j
+      const int k0 = j - 1, k1 = j - 2;
+      f(c0 + 2 + 2 * ch, e, (k0 >= 0 && k0 < kWin) ? k0 : -1, (k1 >= 0 && k1 < kWin) ? k1 : -1);
+    }
+}
+
+__global__ void __launch_bounds__(kTileThreads, kTileCtas)
+    ssim_fwd_tile_kernel(const __grid_constant__ LossParams P, const float* __restrict__ img,
+                         const float* __restrict__ tgt, float* __restrict__ part, float2* __restrict__ bsum) {
+  wait_prior_grid();
+  __shared__ __align__(16) float2 sxy[kHY][kSW];  // (x, y)
+  __shared__ __align__(16) float2 hm[kHY][kTX];   // row sums of (x, y)
+  __shared__ __align__(16) float2 hq[kHY][kTX];   // row sums of (x^2, y^2)
+  __shared__ __align__(16) float hc[kHY][kTX];    // row sums of x y
+  __shared__ float red[2][kTileThreads / 32];
+  const StripAt t = strip_at(P, blockIdx.x);
+  const int W = t.W, H = t.H;
+  load_halo(t, [&](int r, int c, size_t o, bool in) {
+    cp_async4(&sxy[r][c].x, img + o, 0u, in ? 4u : 0u);
+    cp_async4(&sxy[r][c].y, tgt + o, 0u, in ? 4u : 0u);
+  });
+  __syncthreads();
+  // rows: two output columns per work item, (x, y) and (x^2, y^2) in packed pairs
+  for (int it = threadIdx.x; it < kHY * (kTX / 2); it += kTileThreads) {
+    const int r = it / (kTX / 2), c0 = 2 * (it % (kTX / 2));
+    float2 m0 = make_float2(0.0f, 0.0f), m1 = m0, q0 = m0, q1 = m0;
+    float x0 = 0.0f, x1 = 0.0f;
+    float4 w = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    row_taps(c0, [&](int col, int e, int k0, int k1) {
+      if (e == 0) w = *reinterpret_cast<const float4*>(&sxy[r][col]);
+      const float2 v = e == 0 ? make_float2(w.x, w.y) : make_float2(w.z, w.w);
+      const float2 sq = mul2(v, v);
+      const float cr = v.x * v.y;
+      if (k0 >= 0) {
+        m0 = fma2(tap(P, k0), v, m0);
+        q0 = fma2(tap(P, k0), sq, q0);
+        x0 = fmaf(tap(P, k0).x, cr, x0);
+      }
+      if (k1 >= 0) {
+        m1 = fma2(tap(P, k1), v, m1);
+        q1 = fma2(tap(P, k1), sq, q1);
+        x1 = fmaf(tap(P, k1).x, cr, x1);
+      }
+    });
+    *reinterpret_cast<float4*>(&hm[r][c0]) = make_float4(m0.x, m0.y, m1.x, m1.y);
+    *reinterpret_cast<float4*>(&hq[r][c0]) = make_float4(q0.x, q0.y, q1.x, q1.y);
+    *reinterpret_cast<float2*>(&hc[r][c0]) = make_float2(x0, x1);
+  }
+  __syncthreads();
+  // columns: four output rows per thread
+  const int c = threadIdx.x % kTX, r0 = 4 * (threadIdx.x / kTX);
+  float2 am[4], aq[4];
+  float ac[4];
+#pragma unroll
+  for (int o = 0; o < 4; ++o) {
+    am[o] = aq[o] = make_float2(0.0f, 0.0f);
+    ac[o] = 0.0f;
+  }
+#pragma unroll
+  for (int j = 0; j < kWin + 3; ++j) {
+    const float2 m = hm[r0 + j][c], q = hq[r0 + j][c];
+    const float x = hc[r0 + j][c];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      const int k = j - o;
+      if (k < 0 || k >= kWin) continue;
+      am[o] = fma2(tap(P, k), m, am[o]);
+      aq[o] = fma2(tap(P, k), q, aq[o]);
+      ac[o] = fmaf(tap(P, k).x, x, ac[o]);
+    }
+  }
+  float ssum = 0.0f, lsum = 0.0f;
+  const size_t plane = P.plane;
+#pragma unroll
+  for (int o = 0; o < 4; ++o) {
+    const int r = r0 + o;
+    const int gx = t.gx0 + c, gy = t.gy0 + r;
+    if (gx >= W || gy >= H) continue;
+    const float mx = am[o].x, my = am[o].y, exx = aq[o].x, eyy = aq[o].y, exy = ac[o];
+    const float A = 2.0f * mx * my + kC1;
+    const float B = 2.0f * (exy - mx * my) + kC2;
+    const float Cc = mx * mx + my * my + kC1;
+    const float D = (exx - mx * mx) + (eyy - my * my) + kC2;
+    const float icd = __fdividef(1.0f, Cc * D);
+    const float S = A * B * icd;
+    const float dA = B * icd, dB = A * icd, dC = -__fdividef(S, Cc), dD = -__fdividef(S, D);
+    // through A (2 mu_y), B (-2 mu_y), Cc (2 mu_x) and D (-2 mu_x)
+    const float s_mu = 2.0f * (my * (dA - dB) + mx * (dC - dD));
+    const size_t idx = t.base + (size_t)gy * W + gx;
+    part[idx] = s_mu;
+    part[plane + idx] = dD;
+    part[2 * plane + idx] = 2.0f * dB;
+    ssum += S;
+    const float2 xy = sxy[r + kRad][c + kCOff];
+    lsum += fabsf(xy.x - xy.y);
+  }
+  // block sums (fixed shuffle tree, then the warps in order)
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    ssum += __shfl_xor_sync(0xffffffffu, ssum, d);
+    lsum += __shfl_xor_sync(0xffffffffu, lsum, d);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = ssum;
+    red[1][threadIdx.x >> 5] = lsum;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float a = 0.0f, b = 0.0f;
+    for (int w = 0; w < kTileThreads / 32; ++w) {
+      a += red[0][w];
+      b += red[1][w];
+    }
+    bsum[blockIdx.x] = make_float2(a, b);
+  }
+}
+
+__global__ void __launch_bounds__(kTileThreads, kTileCtas)
+    ssim_bwd_tile_kernel(const __grid_constant__ LossParams P, const float* __restrict__ img,
+                         const float* __restrict__ tgt, const float* __restrict__ part, float* __restrict__ dL,
+                         const float2* __restrict__ bsum, float* __restrict__ loss) {
+  wait_prior_grid();
+  __shared__ __align__(16) float2 sp[kHY][kSW];  // (S_mu, S_xx)
+  __shared__ __align__(16) float sc[kHY][kSW];   // S_xy
+  __shared__ __align__(16) float2 hp[kHY][kTX];
+  __shared__ __align__(16) float hs[kHY][kTX];
+  if (blockIdx.x == 0) {
+    loss_reduce<kTileThreads>(P, bsum, loss, reinterpret_cast<float*>(sp));
+    return;
+  }
+  const StripAt t = strip_at(P, blockIdx.x - 1);
+  const int W = t.W, H = t.H;
+  const size_t plane = P.plane;
+  // this thread's four outputs (column c, rows r0 .. r0 + 3): their image and
+  // target values are loaded first, to arrive during the passes
+  const int c = threadIdx.x % kTX, r0 = 4 * (threadIdx.x / kTX);
+  float xo[4], yo[4];
+  size_t io[4];
+  bool ok[4];
+#pragma unroll
+  for (int o = 0; o < 4; ++o) {
+    const int gx = t.gx0 + c, gy = t.gy0 + r0 + o;
+    ok[o] = gx < W && gy < t.H;
+    io[o] = t.base + (size_t)(ok[o] ? gy : 0) * W + (ok[o] ? gx : 0);
+    xo[o] = ok[o] ? img[io[o]] : 0.0f;
+    yo[o] = ok[o] ? tgt[io[o]] : 0.0f;
+  }
+  load_halo(t, [&](int r, int cc, size_t o, bool in) {
+    cp_async4(&sp[r][cc].x, part + o, 0u, in ? 4u : 0u);
+    cp_async4(&sp[r][cc].y, part + plane + o, 0u, in ? 4u : 0u);
+    cp_async4(&sc[r][cc], part + 2 * plane + o, 0u, in ? 4u : 0u);
+  });
+  __syncthreads();
+  for (int it = threadIdx.x; it < kHY * (kTX / 2); it += kTileThreads) {
+    const int r = it / (kTX / 2), c0 = 2 * (it % (kTX / 2));
+    float2 a0 = make_float2(0.0f, 0.0f), a1 = a0;
+    float b0 = 0.0f, b1 = 0.0f;
+    float4 w = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    float2 z = make_float2(0.0f, 0.0f);
+    row_taps(c0, [&](int col, int e, int k0, int k1) {
+      if (e == 0) {
+        w = *reinterpret_cast<const float4*>(&sp[r][col]);
+        z = *reinterpret_cast<const float2*>(&sc[r][col]);
+      }
+      const float2 v = e == 0 ? make_float2(w.x, w.y) : make_float2(w.z, w.w);
+      const float u = e == 0 ? z.x : z.y;
+      if (k0 >= 0) {
+        a0 = fma2(tap(P, k0), v, a0);
+        b0 = fmaf(tap(P, k0).x, u, b0);
+      }
+      if (k1 >= 0) {
+        a1 = fma2(tap(P, k1), v, a1);
+        b1 = fmaf(tap(P, k1).x, u, b1);
+      }
+    });
+    *reinterpret_cast<float4*>(&hp[r][c0]) = make_float4(a0.x, a0.y, a1.x, a1.y);
+    *reinterpret_cast<float2*>(&hs[r][c0]) = make_float2(b0, b1);
+  }
+  __syncthreads();
+  float2 am[4];
+  float ab[4];
+#pragma unroll
+  for (int o = 0; o < 4; ++o) {
+    am[o] = make_float2(0.0f, 0.0f);
+    ab[o] = 0.0f;
+  }
+#pragma unroll
+  for (int j = 0; j < kWin + 3; ++j) {
+    const float2 m = hp[r0 + j][c];
+    const float u = hs[r0 + j][c];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+      const int k = j - o;
+      if (k < 0 || k >= kWin) continue;
+      am[o] = fma2(tap(P, k), m, am[o]);
+      ab[o] = fmaf(tap(P, k).x, u, ab[o]);
+    }
+  }
+  const float n_inv = 1.0f / (3.0f * (float)W * (float)H);
+  const float w1 = P.inv_views * n_inv * (1.0f - P.lam), ws = P.inv_views * n_inv * P.lam;
+#pragma unroll
+  for (int o = 0; o < 4; ++o) {
+    if (!ok[o]) continue;
+    const float x = xo[o], y = yo[o];
+    const float sg = (float)(x > y) - (float)(x < y);
+    // d(1 - SSIM)/dx = -dSSIM/dx
+    dL[io[o]] = w1 * sg - ws * (am[o].x + 2.0f * x * am[o].y + y * ab[o]);
   }
 }
 
@@ -549,6 +812,21 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// Whether the images go by tiles: where they are few (fewer than 2.5 waves of
+// tile CTAs), as a strip's many steps are then a latency that nothing hides, or
+// narrow, as a strip's unused columns cost more than its saved arithmetic
+// gains.  Both kernels by tiles / strips, us: one 256 x 192 image 11 / 24, 400
+// x 301 17 / 26, 800 x 600 36 / 38; two of them (2850 tiles) 58 / 58, three 87
+// / 77; 640 x 360 two (1440) 36 / 38, three (2160) 48 / 46, eight 118 / 89; 256
+// of 64 x 64 (strips of twice the tiles' pixels) 67 / 103, sixteen of 130 x
+// 1000 (1.56 times) 151 / 181, eight of 260 x 1000 (1.30) 138 / 140, eight of
+// 400 x 301 (1.16) 64 / 67, one of 1352 x 1014 83 / 73.  Images of a few rows,
+// most of a tile's empty, go by strips of as few steps: 4000 x 5 15 / 13.
+bool use_tiles(uint64_t tiles, uint64_t strip_px, uint64_t tile_px, int sms) {
+  if (4 * strip_px < tile_px) return false;
+  return 2 * tiles < 5ull * kTileCtas * sms || 4 * strip_px > 5 * tile_px;
+}
+
 int sm_count() {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
@@ -559,43 +837,51 @@ int sm_count() {
 // Sizes and, with P, the blocks of the two kernels on a device of `sms` SMs.
 bool loss_blocks(int32_t n, const int32_t* w, const int32_t* h, int sms, LossParams* P, size_t* ws) {
   if (n < 1 || n > kLossMaxViews || !w || !h) return false;
-  uint64_t pix = 0, sums = 0;
+  uint64_t pix = 0, sums = 0, strip_px = 0, tile_px = 0;
   for (int i = 0; i < n; ++i) {
     if (w[i] < 1 || h[i] < 1 || w[i] > 65535 || h[i] > 65535) return false;
     pix += (uint64_t)w[i] * h[i];
     sums += 3ull * ((w[i] + kSumTile - 1) / kSumTile) * ((h[i] + kSumTile - 1) / kSumTile);
+    strip_px += 3ull * ((w[i] + kLT - 1) / kLT) * kLT * h[i];
+    tile_px += 3ull * ((w[i] + kTX - 1) / kTX) * kTX * ((h[i] + kTY - 1) / kTY) * kTY;
     if (pix > 0x7fffffffull / 3 || sums > 0x7fffffffull) return false;
   }
   *ws = align256(3 * 3 * pix * sizeof(float)) + align256(sums * sizeof(float2));
   if (!P) return true;
-  // The strips' height: a multiple of the step, between kMinRows (each strip
-  // also walks 2 kRad halo rows: 16 and 24 rows took 150 and 148 us for a
-  // training step at 800 x 600, 32 took 147) and kMaxRows, and in between the
-  // least for which all CTAs, the backward's reducing one too, are resident at
-  // once (1920 x 1080 with five strips too many 112 us, so 97); as kMinRows >=
-  // kSumTile there is a block sum for each
-  static_assert(kMinRows >= kSumTile && kMinRows % kLR == 0 && kLT >= kSumTile, "a block sum per strip");
-  uint64_t rows = kMinRows;
-  auto blocks = [&](uint64_t r) {
-    uint64_t k = 1;
-    for (int i = 0; i < n; ++i) k += 3ull * ((w[i] + kLT - 1) / kLT) * ((h[i] + r - 1) / r);
-    return k;
-  };
-  while (rows < kMaxRows && blocks(rows) > (uint64_t)sms * kLossCtas) rows += kLR;
+  if (use_tiles(sums, strip_px, tile_px, sms)) {
+    P->cols = kTX;
+    P->rows = kTY;
+  } else {
+    // The strips' height: a multiple of the step, between kMinRows (each strip
+    // also walks 2 kRad halo rows: 16 and 24 rows took 150 and 148 us for a
+    // training step at 800 x 600, 32 took 147) and kMaxRows, and in between the
+    // least for which all CTAs, the backward's reducing one too, are resident
+    // at once (1920 x 1080 with five strips too many 112 us, so 97); as
+    // kMinRows >= kSumTile there is a block sum for each
+    static_assert(kMinRows >= kSumTile && kMinRows % kLR == 0 && kLT >= kSumTile, "a block sum per strip");
+    uint64_t rows = kMinRows;
+    auto blocks = [&](uint64_t r) {
+      uint64_t k = 1;
+      for (int i = 0; i < n; ++i) k += 3ull * ((w[i] + kLT - 1) / kLT) * ((h[i] + r - 1) / r);
+      return k;
+    };
+    while (rows < kMaxRows && blocks(rows) > (uint64_t)sms * kLossCtas) rows += kLR;
+    P->cols = kLT;
+    P->rows = (int32_t)rows;
+  }
   uint64_t blk = 0, at = 0;
   for (int i = 0; i < n; ++i) {
     LossView& v = P->v[i];
     v.W = w[i];
     v.H = h[i];
-    v.tiles_x = (w[i] + kLT - 1) / kLT;
-    v.tiles = v.tiles_x * (int32_t)((h[i] + rows - 1) / rows);
+    v.tiles_x = (w[i] + P->cols - 1) / P->cols;
+    v.tiles = v.tiles_x * ((h[i] + P->rows - 1) / P->rows);
     v.pix_off = (uint32_t)at;
     v.blk_off = (uint32_t)blk;
     at += (uint64_t)w[i] * h[i];
     blk += 3ull * v.tiles;
   }
   P->n_blocks = (uint32_t)blk;
-  P->rows = (int32_t)rows;
   P->n = n;
   P->plane = 3 * pix;
   return true;
@@ -637,11 +923,13 @@ extern "C" ubs_status ubs_image_loss(int32_t n_views, const int32_t* widths, con
   char* ws = (char*)workspace;
   float* part = (float*)ws;
   float2* bsum = (float2*)(ws + align256(3 * p.plane * sizeof(float)));
-  cudaError_t e = launch_dependent(ssim_fwd_kernel, dim3(p.n_blocks), dim3(kLT), 0, stream, p, image,
-                                   target, part, bsum);
+  const bool tiles = p.cols == kTX;
+  const dim3 block(tiles ? kTileThreads : kLT);
+  cudaError_t e = launch_dependent(tiles ? ssim_fwd_tile_kernel : ssim_fwd_kernel, dim3(p.n_blocks), block, 0, stream,
+                                   p, image, target, part, bsum);
   if (e == cudaSuccess)
-    e = launch_dependent(ssim_bwd_kernel, dim3(p.n_blocks + 1), dim3(kLT), 0, stream, p, image, target,
-                         (const float*)part, dL_dimage, (const float2*)bsum, loss);
+    e = launch_dependent(tiles ? ssim_bwd_tile_kernel : ssim_bwd_kernel, dim3(p.n_blocks + 1), block, 0, stream, p,
+                         image, target, (const float*)part, dL_dimage, (const float2*)bsum, loss);
   return e == cudaSuccess ? UBS_OK : UBS_ERR_CUDA;
 }
 

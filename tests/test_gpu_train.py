@@ -265,3 +265,19 @@ def test_adam_words_across_planes(dev, P):
         assert st == U.UBS_OK
         out.append((raw, act, m, v))
     assert all(torch.equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("large", [2, 3, 5, 16])
+def test_image_loss_forms_over_mixed_sizes(dev, large):
+    """Sizes at the edges of strips and tiles beside enough larger images that
+    the whole goes by strips (of the least height, of a height that fits the
+    GPU, of the greatest), and, with two of them, by tiles: losses and gradients
+    against the float64 reference, with the bounds of the larger cases."""
+    sizes = [(128, 16), (129, 17), (127, 15), (31, 200), (5, 97), (1, 1), (257, 64), (128, 33), (384, 36), (640, 97)]
+    test_image_loss_at_strip_edges(dev, sizes + [(640, 352)] * large)
+
+
+@pytest.mark.parametrize("sizes", [[(4000, 5)], [(300, 6), (129, 4)], [(1, 1)]])
+def test_image_loss_of_a_few_rows(dev, sizes):
+    """Images of fewer rows than a strip's step count takes, alone."""
+    test_image_loss_at_strip_edges(dev, sizes)
