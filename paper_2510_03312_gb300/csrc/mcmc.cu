@@ -42,7 +42,7 @@ namespace ubs {
 namespace {
 
 constexpr int kMcBlock = 1024;  // elements per scan block
-constexpr int kMcChunk = 64;    // elements per chunk of the in-block search: two per lane
+constexpr int kMcChunk = 64;    // elements per chunk of the in-block search: four per lane of a half-warp
 constexpr int kMcChunks = kMcBlock / kMcChunk;  // chunks per block
 constexpr unsigned kMcCopyRow = 152;            // blocks per plane of the copy kernel
 constexpr int kMcThreads = 256;
@@ -173,30 +173,40 @@ __device__ __forceinline__ float cloned_opacity(float o, uint32_t n) {
   return 1.0f - powf(1.0f - o, 1.0f / (float)(n + 1));
 }
 
-// inclusive sum over the lanes up to this one
-__device__ __forceinline__ unsigned long long warp_incl_scan(unsigned long long x) {
-  const int lane = threadIdx.x & 31;
+// inclusive sum over the lanes of a half-warp up to this one
+__device__ __forceinline__ unsigned long long half_incl_scan(unsigned long long x) {
+  const int lane = threadIdx.x & 15;
 #pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const unsigned long long y = __shfl_up_sync(0xffffffffu, x, d);
+  for (int d = 1; d < 16; d <<= 1) {
+    const unsigned long long y = __shfl_up_sync(0xffffffffu, x, d, 16);
     if (lane >= d) x += y;
   }
   return x;
 }
 
-// A block draws for the dead of its kMcBlock slots: it lists them in shared
+// A block draws for the dead of its `slots` slots: it lists them in shared
 // memory, each thread then takes a listed slot and finds the block of
 // primitives its draw falls in (every stride-th block offset is staged in
 // shared memory; at most two steps' worth of offsets are then read from
-// global memory for scenes of up to 4M primitives), and each warp finishes
-// its slots one after the other with all lanes: the chunk sums of the block,
-// then the chunk's weights, two dependent loads a slot.
+// global memory for scenes of up to 4M primitives), and each half-warp
+// finishes slots one after the other: the chunk sums of the block, a lane
+// each, then the chunk's weights, four a lane, two dependent loads a slot.
+// Where many of the slots are dead this chain is the call's time (a whole
+// warp a slot, with wider scans: 1M primitives, K = 14, 95% dead 398 us, 304
+// so; 20% 174, 155), so a CTA takes 1024 slots only in scenes that give two
+// CTAs an SM that way, and down to 64 in smaller ones: 100K primitives, 20%
+// dead 46 us with 1024, 29 with 256 (5% 32, 25); 5000, 20% 33, 20 with 64.
 constexpr uint32_t kMcOffs = 1024;  // staged block offsets
+inline int draw_slots(int64_t P) {
+  int slots = kMcBlock;
+  while (slots > 64 && (P + slots - 1) / slots < 152 * 2) slots /= 2;
+  return slots;
+}
 __global__ void __launch_bounds__(kMcThreads)
     mcmc_draw_kernel(const float* __restrict__ op, int64_t P, float thr, const unsigned long long* __restrict__ rnd,
                      const unsigned long long* __restrict__ csum, const unsigned long long* __restrict__ boff,
                      uint32_t nb, uint32_t* __restrict__ counts, int32_t* __restrict__ src,
-                     int32_t* __restrict__ list, McHeader* hdr) {
+                     int32_t* __restrict__ list, McHeader* hdr, int slots) {
   wait_prior_grid();
   __shared__ unsigned long long s_off[kMcOffs];
   __shared__ int32_t s_slot[kMcBlock];
@@ -211,8 +221,9 @@ __global__ void __launch_bounds__(kMcThreads)
   __syncthreads();
 #pragma unroll
   for (int e = 0; e < kMcBlock / kMcThreads; ++e) {
-    const int64_t j = (int64_t)blockIdx.x * kMcBlock + e * kMcThreads + threadIdx.x;
-    const bool dead = j < P && is_dead(op[j], thr);
+    const int at_block = e * kMcThreads + threadIdx.x;
+    const int64_t j = (int64_t)blockIdx.x * slots + at_block;
+    const bool dead = at_block < slots && j < P && is_dead(op[j], thr);
     const unsigned all = __ballot_sync(0xffffffffu, dead);
     uint32_t at = 0;
     if (lane == 0 && all) at = atomicAdd(&s_n, (uint32_t)__popc(all));
@@ -247,30 +258,34 @@ __global__ void __launch_bounds__(kMcThreads)
       }
       r -= boff[lo];
     }
-    const unsigned act = __ballot_sync(0xffffffffu, on);
+    const int n_on = __popc(__ballot_sync(0xffffffffu, on));  // the first lanes
     int32_t from = -1;
-    for (unsigned rest = act; rest != 0; rest &= rest - 1) {
-      const int l = __ffs(rest) - 1;
-      unsigned long long rr = __shfl_sync(0xffffffffu, r, l);
-      const uint32_t b = __shfl_sync(0xffffffffu, lo, l);
-      // the block's first chunk whose inclusive sum exceeds rr
-      const unsigned long long cs = lane < kMcChunks ? csum[(size_t)b * kMcChunks + lane] : 0ull;
-      unsigned long long x = warp_incl_scan(cs);
-      const int ch = __ffs(__ballot_sync(0xffffffffu, x > rr)) - 1;  // some chunk does: r < total
-      rr -= __shfl_sync(0xffffffffu, x - cs, ch);
-      // and that chunk's first primitive, in its first or second half
-      const int64_t p = (int64_t)b * kMcBlock + ch * kMcChunk + lane;
-      const uint32_t q0 = p < P ? weight_of(op[p], thr) : 0u, q1 = p + 32 < P ? weight_of(op[p + 32], thr) : 0u;
-      x = warp_incl_scan(q0);
-      unsigned over = __ballot_sync(0xffffffffu, x > rr);
-      int at = __ffs(over) - 1;
-      if (over == 0) {  // warp-uniform
-        rr -= __shfl_sync(0xffffffffu, x, 31);
-        x = warp_incl_scan(q1);
-        over = __ballot_sync(0xffffffffu, x > rr);
-        at = 31 + __ffs(over);
+    const int half = lane >> 4, sub = lane & 15;
+    for (int l = 0; l < n_on; l += 2) {
+      const int own = min(l + half, n_on - 1);  // this half-warp's slot
+      unsigned long long rr = __shfl_sync(0xffffffffu, r, own);
+      const uint32_t b = __shfl_sync(0xffffffffu, lo, own);
+      // the block's first chunk whose inclusive sum exceeds rr (some chunk's does: r < total)
+      const unsigned long long cs = csum[(size_t)b * kMcChunks + sub];
+      unsigned long long x = half_incl_scan(cs);
+      const int ch = __ffs((__ballot_sync(0xffffffffu, x > rr) >> (16 * half)) & 0xffffu) - 1;
+      rr -= __shfl_sync(0xffffffffu, x - cs, ch, 16);
+      // and that chunk's first primitive: four to a lane
+      const int64_t p = (int64_t)b * kMcBlock + ch * kMcChunk + 4 * sub;
+      unsigned long long q[4], sum = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        sum += p + k < P ? weight_of(op[p + k], thr) : 0u;
+        q[k] = sum;
       }
-      if (lane == l) from = (int32_t)((int64_t)b * kMcBlock + ch * kMcChunk + at);
+      x = half_incl_scan(sum);
+      const int f = __ffs((__ballot_sync(0xffffffffu, x > rr) >> (16 * half)) & 0xffffu) - 1;
+      rr -= x - sum;  // in lane f, what is left for its four
+      const int at = 4 * sub + (rr < q[0] ? 0 : rr < q[1] ? 1 : rr < q[2] ? 2 : 3);
+      const int64_t g = (int64_t)b * kMcBlock + ch * kMcChunk + __shfl_sync(0xffffffffu, at, f, 16);
+      const int32_t v0 = __shfl_sync(0xffffffffu, (int32_t)g, 0), v1 = __shfl_sync(0xffffffffu, (int32_t)g, 16);
+      if (lane == l) from = v0;
+      if (lane == l + 1) from = v1;  // n_on odd: lane l + 1 holds no slot
     }
     if (on) {
       src[s_slot[i]] = from;
@@ -364,14 +379,18 @@ extern "C" ubs_status ubs_mcmc_relocate(int32_t K, int64_t P, int32_t opacity_ro
   const float* op = act + (size_t)opacity_row * P;
   const unsigned grid = (unsigned)((P + kMcThreads - 1) / kMcThreads);
   McPlanes pl{K, opacity_row};
+  const int slots = draw_slots(P);
   cudaError_t e = launch_dependent(mcmc_weights_kernel, dim3(L.nb), dim3(kMcThreads), 0, stream, op, P,
                                    dead_threshold, csum, boff, counts, src);
   if (e == cudaSuccess) e = launch_dependent(mcmc_scan_kernel, dim3(1), dim3(1024), 0, stream, boff, L.nb, hdr);
   if (e == cudaSuccess)
-    e = launch_dependent(mcmc_draw_kernel, dim3(L.nb), dim3(kMcThreads), 0, stream, op, P, dead_threshold,
-                         (const unsigned long long*)rand, (const unsigned long long*)csum,
-                         (const unsigned long long*)boff, L.nb, counts, src, list, hdr);
-  const unsigned row = grid < kMcCopyRow ? grid : kMcCopyRow;
+    e = launch_dependent(mcmc_draw_kernel, dim3((unsigned)((P + slots - 1) / slots)), dim3(kMcThreads), 0, stream, op,
+                         P, dead_threshold, (const unsigned long long*)rand, (const unsigned long long*)csum,
+                         (const unsigned long long*)boff, L.nb, counts, src, list, hdr, slots);
+  // a CTA a plane per 1024 slots (most hold no dead one: 100K primitives, K = 36,
+  // 1% dead 27 us with one per 256, 25 so), where that leaves some for each plane
+  const unsigned least = grid < 16 ? grid : 16, most = L.nb < kMcCopyRow ? L.nb : kMcCopyRow;
+  const unsigned row = most < least ? least : most;
   if (e == cudaSuccess)
     e = launch_dependent(mcmc_copy_kernel, dim3(row, (unsigned)K), dim3(kMcThreads), 0, stream, pl, P, act, raw,
                          (const int32_t*)src, (const int32_t*)list, (const McHeader*)hdr);

@@ -113,3 +113,48 @@ def test_draw_search_at_its_level_edges(dev, P, dead_frac):
     moved = dead | (copies > 0)
     assert np.array_equal(m[0].cpu().numpy(), np.where(moved, 0.0, 1.0).astype(np.float32))
     assert np.array_equal(v[0].cpu().numpy(), np.where(moved, 0.0, 1.0).astype(np.float32))
+
+
+@pytest.mark.parametrize("P,dead_frac", [(31, 0.5), (63, 0.5), (64, 0.5), (65, 0.5), (1023, 0.3), (1024, 0.95),
+                                         (1025, 0.95), (19_455, 0.2), (19_457, 0.95), (311_295, 0.95),
+                                         (311_297, 0.05), (1024 * 1024, 0.02), (3 * 1024 * 1024 + 1, 0.01)])
+def test_draw_at_chunk_and_block_edges(dev, P, dead_frac):
+    """The draw at the edges of its chunks of 64 and blocks of 1024
+    primitives, of the slots a CTA takes (64 to 1024 by the scene's size) and
+    of the staged block offsets (every one up to 1M primitives, then every
+    second and fourth), with few and with nearly all slots dead."""
+    test_draw_search_at_its_level_edges(dev, P, dead_frac)
+
+
+@pytest.mark.parametrize("P", [64, 1024, 4096, 1500 * 1024])
+@pytest.mark.parametrize("live", ["last_of_four", "second_half", "one_per_chunk", "one_per_block", "last_block"])
+def test_draw_among_few_live_primitives(dev, P, live):
+    """Weights in one place of each group the draw searches: the last of a
+    lane's four, the second half of a chunk, one primitive a chunk or a block,
+    and the last block only (whole staged steps without weight before it): the
+    sources against the cumulative weights by definition, bit for bit."""
+    import ctypes
+
+    from paper_2510_03312_gb300 import ubs as U
+    rng = np.random.default_rng(P)
+    i = np.arange(P)
+    on = {"last_of_four": i % 4 == 3, "second_half": i % 64 >= 32, "one_per_chunk": i % 64 == (i // 64 * 7) % 64,
+          "one_per_block": i % 1024 == min(P, 1024) - 1, "last_block": i >= P - min(P // 2, 1024)}[live]
+    o = np.where(on, rng.uniform(0.006, 1.0, P), 0.0).astype(np.float32)
+    rand = rng.integers(0, 2 ** 63, size=P, dtype=np.uint64) * np.uint64(2) + np.uint64(1)
+    w = np.where(on, np.floor(o.astype(np.float64) * 2 ** 24), 0).astype(np.uint64)
+    cum = np.cumsum(w, dtype=np.uint64)
+    rand[:2] = 0, cum[-1] - np.uint64(1)  # the first and the last unit of weight
+    want = np.where(on, -1, np.searchsorted(cum, rand % cum[-1], side="right")).astype(np.int32)
+    act, raw, m, v = (torch.tensor(a, device=dev)[None].contiguous() for a in (o, 0 * o, 0 * o, 0 * o))
+    rnd = torch.tensor(rand.view(np.int64), device=dev)
+    src = torch.empty(P, dtype=torch.int32, device=dev)
+    nrel = torch.zeros(1, dtype=torch.int64, device=dev)
+    n = U.ubs_mcmc_workspace_size(P)
+    ws = torch.empty(n + 256, dtype=torch.uint8, device=dev)
+    st = U.ubs_mcmc_relocate(1, P, 0, 0.005, act.data_ptr(), raw.data_ptr(), m.data_ptr(), v.data_ptr(),
+                             rnd.data_ptr(), src.data_ptr(), nrel.data_ptr(), (ws.data_ptr() + 255) // 256 * 256, n,
+                             ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == U.UBS_OK
+    assert np.array_equal(src.cpu().numpy(), want)
+    assert int(nrel.item()) == int((~on).sum())
