@@ -281,3 +281,37 @@ def test_image_loss_forms_over_mixed_sizes(dev, large):
 def test_image_loss_of_a_few_rows(dev, sizes):
     """Images of fewer rows than a strip's step count takes, alone."""
     test_image_loss_at_strip_edges(dev, sizes)
+
+
+@pytest.mark.parametrize("P", [4, 8, 1000, 4096])
+def test_adam_words_within_planes(dev, P):
+    """P a multiple of four: words that lie within a plane, with the noise read
+    by words too, against the same step with the noise off the 16-byte boundary
+    (words, the noise by elements) and with every buffer off it (elements), bit
+    for bit; with noise and without."""
+    import ctypes
+
+    from paper_2510_03312_gb300 import train as TR
+    from paper_2510_03312_gb300 import ubs as U
+    table = TR.plane_table(6, S.ROT_SKEW1, TR.TrainConfig())
+    K = len(table)
+    g = torch.Generator(device=dev).manual_seed(P)
+    src = [torch.randn(K * P, generator=g, device=dev) * s for s in (0.5, 1.0, 1e-2, 1e-3)] + \
+          [torch.rand(K * P, generator=g, device=dev) * 1e-5, torch.randn(3 * P, generator=g, device=dev) * 1e-3]
+    for noisy in (True, False):
+        planes = (U.ubs_adam_plane * K)()
+        for k, (lr, a, l1, row) in enumerate(table):
+            planes[k].lr, planes[k].activation, planes[k].l1_weight = lr, a, l1
+            planes[k].noise_row = row if noisy else -1
+        out = []
+        for off, off_noise in ((0, 0), (0, 1), (1, 1)):
+            raw, act, grad, m, v = [torch.cat([torch.zeros(off, device=dev), s])[off:] for s in src[:5]]
+            noise = torch.cat([torch.zeros(off_noise, device=dev), src[5]])[off_noise:]
+            st = U.ubs_adam_step(K, P, planes, U.ubs_adam_config(0.9, 0.999, 1e-15, 7, 1.0), raw.data_ptr(),
+                                 act.data_ptr(), grad.data_ptr(), m.data_ptr(), v.data_ptr(),
+                                 noise.data_ptr() if noisy else None,
+                                 ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+            assert st == U.UBS_OK
+            out.append((raw, act, m, v))
+        for other in out[1:]:
+            assert all(torch.equal(a, b) for a, b in zip(out[0], other))
