@@ -10,6 +10,7 @@ diagonal of L_q = exp(raw), everything else the identity.
 """
 from __future__ import annotations
 
+import ctypes
 from dataclasses import dataclass
 
 import numpy as np
@@ -131,9 +132,7 @@ class Adam:
         for k, (lr, a, l1, row) in enumerate(self.table):
             self._planes[k].lr, self._planes[k].activation = lr, a
             self._planes[k].l1_weight, self._planes[k].noise_row = l1, row
-        self._planes_quiet = (U.ubs_adam_plane * K)(*self._planes)  # for steps without noise
-        for k in range(K):
-            self._planes_quiet[k].noise_row = -1
+        self._planes_quiet = (U.ubs_adam_plane * K)()  # of a step without noise: filled from _planes by each
 
     def step(self, grad: torch.Tensor, noise: torch.Tensor | None = None):
         """One step with dL/d(activated params) ``grad``; ``noise`` [3, P] is the
@@ -146,7 +145,11 @@ class Adam:
         self.step_count += 1
         cfg = U.ubs_adam_config(self.tc.beta1, self.tc.beta2, self.tc.eps, self.step_count,
                                 self.tc.lambda_eps if noise is not None else 0.0)
-        planes = self._planes if noise is not None else self._planes_quiet
+        planes = self._planes
+        if noise is None:  # the plane table as it is now (its rates may have been changed), with no noise
+            planes = self._planes_quiet
+            ctypes.memmove(planes, self._planes, ctypes.sizeof(planes))
+            np.frombuffer(planes, np.int32).reshape(self.K, -1)[:, 3] = -1  # noise_row
         st = U.ubs_adam_step(self.K, self.P, planes, cfg, self.raw.data_ptr(), self.act.data_ptr(),
                              grad.data_ptr(), self.m.data_ptr(), self.v.data_ptr(),
                              noise.data_ptr() if noise is not None else None,

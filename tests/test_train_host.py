@@ -71,3 +71,35 @@ def test_checkpoint_round_trip(tmp_path):
     other = TR.Adam(S.make_scene(9, 3, 40), torch.tensor(S.make_scene(9, 3, 40).params))
     with pytest.raises(ValueError):
         TR.load_checkpoint(path, [other])
+
+
+def test_adam_steps_take_the_plane_table_as_it_is(monkeypatch):
+    """A rate changed in the plane table between steps (a schedule) reaches the
+    next step with noise and without, of a copied optimiser too; a step without
+    noise gives no plane a noise row and leaves the table's own rows."""
+    import copy
+    from types import SimpleNamespace
+
+    sc = S.make_scene(9, 6, 40)
+    a = copy.deepcopy(TR.Adam(sc, torch.tensor(sc.params)))
+    seen = []
+
+    def step(K, P, planes, cfg, *args):
+        seen.append([(p.lr, p.activation, p.l1_weight, p.noise_row) for p in planes])
+        return U.UBS_OK
+
+    monkeypatch.setattr(TR.U, "ubs_adam_step", step)
+    monkeypatch.setattr(TR, "check_tensor", lambda *args, **kw: None)
+    monkeypatch.setattr(TR, "current_stream", lambda: None)
+    a.act = SimpleNamespace(device=SimpleNamespace(type="cuda"), data_ptr=lambda: 0)
+    g = torch.zeros(a.K, a.P)
+    for lr in (0.25, 0.125):
+        a._planes[2].lr = lr
+        for noise in (None, torch.zeros(3, a.P)):
+            a.step(g, noise)
+            got = seen[-1]
+            assert got[2][0] == lr
+            assert [x[:3] for x in got] == [(p.lr, p.activation, p.l1_weight) for p in a._planes]
+            rows = [x[3] for x in a.table]
+            assert [x[3] for x in got] == (rows if noise is not None else [-1] * a.K)
+    assert [p.noise_row for p in a._planes] == [x[3] for x in a.table]
