@@ -261,3 +261,110 @@ def test_few_tiles_match_many(tile):
         px = v.width * v.height
         got.append((r.image[:3 * px].clone(), r.export(U.EXPORT_FINAL_T)[:px].clone(), r.export(U.EXPORT_LAST)[:px].clone()))
     assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+def _planned_segment(r, lists):
+    """Entries per segment that the split form plans for these list lengths
+    (uint32 per tile), restated from the rule: the shortest of 128 (or the
+    blend's batch of 256 entries for tiles over 256 pixels) and its doublings
+    up to 2048 of which there are at most 16 per SM and whose state the
+    workspace holds."""
+    def up(x):
+        return (x + 255) // 256 * 256
+    px = int(r.cfg.tile_w) * int(r.cfg.tile_h)
+    nt, cap = r.n_tiles(), r.capacity
+    ms = cap // 2048 + 1
+    aside = up(16 * ms) + up(4 * nt) + up(2 * ms * px * 32) + up(8 * ms) + 2 * up(4 * ms)
+    room = up(8 * r.n_pix) + aside - up(16 * ms) - up(4 * nt) - up(4 * ms * px) - up(4 * ms)
+    slots = min((room - 1024) // (20 * px + 8), cap // 128 + ms)
+    safe = 128
+    while safe < 2048 and cap // safe + ms > slots:
+        safe *= 2
+    chunks = int(sum(-(-int(n) // 512) for n in lists if n > 512))
+    length = 128 if px <= 256 else 256
+    while length < 2048 and (chunks * 512 > 152 * 16 * length or
+                             (length < safe and chunks * max(1, 512 // length) > slots)):
+        length *= 2
+    return length
+
+
+def _used_segment(r, lists):
+    """Entries per segment that the kernels used: the split tiles' table
+    (tile, first slot, segments, first extra segment) found in the workspace
+    by its tiles."""
+    tiles = np.flatnonzero(lists > 2048)
+    off = r.ws_ptr - r._ws.data_ptr()
+    words = r._ws[off:off + r.ws_bytes // 4 * 4].cpu().numpy().view(np.uint32)
+    found = set()
+    for o in range(0, words.size - 4 * tiles.size, 64):  # on 256-byte boundaries
+        if words[o] not in tiles:
+            continue
+        t = words[o:o + 4 * tiles.size].reshape(-1, 4)
+        if not np.array_equal(np.sort(t[:, 0]), tiles):
+            continue
+        for length in (128, 256, 512, 1024, 2048):
+            if np.array_equal(t[:, 2], -(-lists[t[:, 0]].astype(np.int64) // length)):
+                found.add(length)
+    assert len(found) == 1, found
+    return found.pop()
+
+
+def _split_against_unsplit(sc, view, tile, capacity):
+    """Renders in both forms: the images within 1e-5, the gradients within 1e-3
+    of their plane's largest and the lists bit for bit; returns the split
+    form's rasterizer and its list lengths."""
+    got = {}
+    for split in (False, True):
+        r = raster.Rasterizer([raster.DeviceScene.from_scene(sc, device="cuda")], [view],
+                              S.RasterConfig(tile_w=tile[0], tile_h=tile[1], split_lists=split),
+                              capacity=capacity, device="cuda")
+        for _ in range(2):  # the second on the segment state the first left
+            r.preprocess()
+            r.bin_sort()
+            img = r.render_fwd().clone()
+        st = r.status()
+        assert st.status == 0
+        start = r.export(U.EXPORT_TILE_START).clone()
+        inst = r.export(U.EXPORT_INSTANCES)[:int(st.instances)].clone()
+        lists = torch.diff(start).cpu().numpy().astype(np.uint32)
+        length = (_planned_segment(r, lists), _used_segment(r, lists)) if split else None
+        dL = torch.sin(torch.arange(img.numel(), device="cuda")) / img.numel()
+        got[split] = img, r.backward(dL)[0].clone(), start, inst
+    assert torch.equal(got[True][2], got[False][2]) and torch.equal(got[True][3], got[False][3])
+    assert (got[True][0] - got[False][0]).abs().max() <= 1e-5
+    worst = ((got[True][1] - got[False][1]).abs().amax(1) / got[False][1].abs().amax(1).clamp(min=1e-30)).max()
+    assert worst <= 1e-3, float(worst)
+    assert length[0] == length[1], length
+    return length[1], lists
+
+
+@pytest.mark.parametrize("tile,length", [((8, 8), 256), ((16, 16), 512), ((16, 32), 512), ((32, 32), 1024)])
+def test_split_segments_of_a_tight_workspace(tile, length):
+    """One long list and a capacity that just holds it: the workspace has state
+    for few segments, and they are longer than the shortest."""
+    n = 9000
+    rng = np.random.default_rng(n)
+    sc = S.make_scene(n, 3, n, scale_range=(0.001, 0.002), rng=rng)
+    sc.plane("mean_x")[:] = (0.0005 * rng.uniform(-1.0, 1.0, (3, n))).astype(np.float32)
+    sc.plane("opacity")[:] = rng.choice([0.005, 0.02, 0.1], n).astype(np.float32)
+    v = S.make_view(np.eye(3), np.array([0.0, 0.0, 4.0]), 75, 71)  # the stack's mean in one tile, whatever its shape
+    used, lists = _split_against_unsplit(sc, v, tile, capacity=n)
+    assert used == length and lists.max() == n == lists.sum()
+
+
+@pytest.mark.parametrize("n,size,length,joined", [(4500, (96, 64), 256, True), (20000, (64, 48), 512, True),
+                                                  (8000, (128, 96), 1024, False), (20000, (96, 64), 1024, False)])
+def test_split_segments_of_many_long_lists(n, size, length, joined):
+    """Every tile's list is long: more entries than segments of the shortest
+    length may number, so that they are longer though the workspace has state
+    for more, and lists over 4096 entries joined by rank up to 2048 chunks of
+    512 and merged in rounds beyond."""
+    rng = np.random.default_rng(n)
+    sc = S.make_scene(n, 3, n, scale_range=(8.0, 12.0), rng=rng)
+    sc.plane("mean_x")[:] = rng.uniform(-0.3, 0.3, (3, n)).astype(np.float32)
+    sc.plane("opacity")[:] = rng.choice([0.006, 0.02], n, p=[0.97, 0.03]).astype(np.float32)
+    v = S.make_view(np.eye(3), np.array([0.0, 0.0, 4.0]), *size)
+    used, lists = _split_against_unsplit(sc, v, (8, 8), capacity=3_000_000)
+    assert used == length and (lists > 2048).all() and lists.max() > 4096
+    chunks = int((-(-lists.astype(np.int64) // 512)).sum())
+    assert (chunks <= 2048) == joined, chunks
