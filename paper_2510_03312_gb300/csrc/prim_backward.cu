@@ -30,38 +30,35 @@ __device__ __forceinline__ void load_prim_b(const SceneDev& sc, int64_t p, PrimI
   }
 }
 
-// N = 3 (C = 0) is held to 72 registers (7 CTAs per SM): G2 is bound by
-// memory latency and gains more from occupancy than it loses to a few spills
-// to L1 (63.5 us unbounded, 53.7 at 6 CTAs, 51.9 at 7 on the 1M-primitive
-// view; 8 gained nothing more); the larger query dimensions would spill too
-// much
-template <int C>
-__global__ void __launch_bounds__(128, C == 0 ? 7 : 1) prim_backward_kernel(SceneDev sc, SceneGradDev gr, ViewList vl,
-                                                            const ViewDev* __restrict__ views, CfgDev cfg,
-                                                            const uint32_t* __restrict__ tiles,
-                                                            const float4* __restrict__ g2d) {
+// Scenes of N = 3 with one view: a thread per primitive; most are drawn, and an
+// undrawn one costs little.  Held to 72 registers (7 CTAs per SM): bound by
+// memory latency, it gains more from occupancy than it loses to a few spills to
+// L1 (63.5 us unbounded, 53.7 at 6 CTAs, 51.9 at 7 on the 1M-primitive view; 8
+// gained nothing more).
+__global__ void __launch_bounds__(128, 7) prim_backward_kernel(SceneDev sc, SceneGradDev gr, int view,
+                                                               const ViewDev* __restrict__ views, CfgDev cfg,
+                                                               const uint32_t* __restrict__ tiles,
+                                                               const float4* __restrict__ g2d) {
   wait_prior_grid();
-  extern __shared__ ViewDev s_views[];
-  for (int i = threadIdx.x; i < vl.n; i += blockDim.x) s_views[i] = views[vl.idx[i]];
+  __shared__ ViewDev s_view;
+  if (threadIdx.x == 0) s_view = views[view];
   __syncthreads();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= sc.P) return;
-  PrimIn<C> in;
-  load_prim_b<C>(sc, p, in);
-  PrimVI<C> vi;
-  prim_stage<C>(in, sc.rot_mode, vi);
-  PrimAcc<C> acc;
-  acc_zero<C>(acc);
-  for (int k = 0; k < vl.n; ++k) {
-    const ViewDev& v = s_views[k];
-    const uint32_t r = v.rec_off + (uint32_t)p;
-    if (tiles[r] == 0) continue;
+  PrimIn<0> in;
+  load_prim_b<0>(sc, p, in);
+  PrimVI<0> vi;
+  prim_stage<0>(in, sc.rot_mode, vi);
+  PrimAcc<0> acc;
+  acc_zero<0>(acc);
+  const uint32_t r = s_view.rec_off + (uint32_t)p;
+  if (tiles[r] != 0) {
     const float4 a = g2d[3 * (size_t)r], b = g2d[3 * (size_t)r + 1], c = g2d[3 * (size_t)r + 2];
     const float g[10] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y};
-    prim_backward_view<C>(in, vi, v, cfg, g, acc);
+    prim_backward_view<0>(in, vi, s_view, cfg, g, acc);
   }
-  PrimGrad<C> out;
-  prim_backward_final<C>(in, vi, sc.rot_mode, acc, out);
+  PrimGrad<0> out;
+  prim_backward_final<0>(in, vi, sc.rot_mode, acc, out);
   const int64_t P = sc.P;
   // written, or added to the caller's running sum (UBS_FLAG_ACCUMULATE_GRADS)
   const bool add = (cfg.flags & 4) != 0;
@@ -70,16 +67,10 @@ __global__ void __launch_bounds__(128, C == 0 ? 7 : 1) prim_backward_kernel(Scen
   const int nr = sc.rot_mode == 0 ? 4 : 3;
   for (int i = 0; i < nr; ++i) put(gr.rot + i * P + p, out.rot[i]);
   for (int i = 0; i < 3; ++i) put(gr.scale_x + i * P + p, out.s[i]);
-  for (int i = 0; i < 1 + C; ++i) put(gr.b + i * P + p, out.b[i]);
+  put(gr.b + p, out.b[0]);
   put(gr.opacity + p, out.o);
   for (int i = 0; i < 3; ++i) put(gr.rgb + i * P + p, out.rgb[i]);
-  if constexpr (C > 0) {
-    for (int i = 0; i < C; ++i) put(gr.mean_q + i * P + p, out.mq[i]);
-    for (int i = 0; i < 3 * C; ++i) put(gr.L_qx + i * P + p, out.lqx[i]);
-    for (int i = 0; i < C * (C + 1) / 2; ++i) put(gr.L_q + i * P + p, out.lq[i]);
-  }
 }
-
 
 // Scenes with query dimensions and one view: one CTA per `prims` consecutive
 // primitives.  It lists those the view draws (their visibility bits) in shared
@@ -195,7 +186,7 @@ __global__ void __launch_bounds__(kPbThreads, C == 3 ? 4 : 1) prim_backward_draw
 }
 
 // Zeroes one scene's gradient planes (the primitives that no view sees keep
-// these zeros; the others are overwritten by prim_backward_kernel).
+// these zeros; the others are overwritten by prim_backward_listed_kernel).
 __global__ void __launch_bounds__(256) zero_scene_grads_kernel(SceneGradDev gr, int64_t P, int C, int nr) {
   wait_prior_grid();
   const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -301,9 +292,9 @@ cudaError_t launch_prim_backward(const SceneDev& sc, const SceneGradDev& g, cons
     }
     return e != cudaSuccess ? e : cudaGetLastError();
   }
-  if (vl.n == 1) {  // N = 3: most primitives are drawn and an undrawn one costs little; every one, directly
-    e = launch_dependent(prim_backward_kernel<0>, dim3((unsigned)nblk), dim3(threads), smem, st, sc, g, vl, views,
-                         cfg, tiles, g2d);
+  if (vl.n == 1) {
+    e = launch_dependent(prim_backward_kernel, dim3((unsigned)nblk), dim3(threads), 0, st, sc, g, (int)vl.idx[0],
+                         views, cfg, tiles, g2d);
     return e != cudaSuccess ? e : cudaGetLastError();
   }
   // several views (or none: an empty list): the listed primitives, the others
