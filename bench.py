@@ -693,7 +693,7 @@ def bench_deep_tile(dev, steps=5, warmup=2):
     """The deep-tile workload (a dense cluster of 60K faint primitives inside
     a few tiles, in front of a 300K-primitive sparse view, 1600x1060): one
     fwd+bwd step with the tile lists blended whole (grid form) and split into
-    segments of 2048 entries merged with the over operator (split form)."""
+    segments merged with the over operator (split form)."""
     import torch
 
     from dataclasses import replace

@@ -92,8 +92,9 @@ enum {
   UBS_FLAG_PERSISTENT = 8, /* the blend kernels run as persistent grids (one CTA per resident
                               slot) that take tiles or 8x8 blocks from a counter in the same order,
                               instead of one CTA per tile or block; the results are the same */
-  UBS_FLAG_SPLIT_LISTS = 16, /* tile lists longer than 2048 entries are split into segments of 128 to
-                               2048 entries (as short as their number and the workspace allow)
+  UBS_FLAG_SPLIT_LISTS = 16, /* tile lists longer than 2048 entries are split into segments of 128
+                               (tiles over 256 pixels: 256) to 2048 entries, as short as their
+                               number and the workspace allow,
                                blended by separate CTAs and merged front to back with the over
                                operator (C = C_1 + T_1 C_2, T = T_1 T_2), walking a segment again
                                for the pixels whose transmittance falls below T_min inside it; the

@@ -125,9 +125,9 @@ struct Layout {
 // Tiles whose lists are longer than kSplitMin entries are split when
 // UBS_FLAG_SPLIT_LISTS is set, into segments of kSegMin (or the blend's batch,
 // where that is longer), 2, 4, .. times that, up to kSplitMin entries: the
-// shortest of which the workspace holds the state, which split_plan_kernel
-// finds from the number of long lists' sort chunks (Header::n_long) and
-// leaves in ctr[kCtrSegLen].
+// shortest of which there are few enough and the workspace holds the state,
+// which split_plan_kernel finds from the number of the sort's chunks of lists
+// over kSortChunk entries (Header::n_long) and leaves in ctr[kCtrSegLen].
 constexpr uint32_t kSplitMin = 2048;
 constexpr uint32_t kSegMin = 128;
 constexpr uint32_t kSegEnded = 0x80000000u;  // flag beside the last contributor (a position below 2^31)

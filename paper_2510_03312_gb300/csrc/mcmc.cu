@@ -31,7 +31,7 @@
 // copy kernel keeps each grid row in one plane and gives a listed slot to
 // each lane, and the moments are zeroed in primitive order, where neighbours
 // share requests.  P = 1M, K = 15, 5% dead, states larger than L2: 208 ->
-// 108 us a call (draw 52 -> 22, copies and moments 151 -> 58; a thread per
+// 100 us a call (draw 52 -> 20, copies and moments 151 -> 59; a thread per
 // slot, most lanes idle, copied and zeroed all planes before).
 #include <math.h>
 
@@ -192,7 +192,7 @@ __device__ __forceinline__ unsigned long long half_incl_scan(unsigned long long 
 // finishes slots one after the other: the chunk sums of the block, a lane
 // each, then the chunk's weights, four a lane, two dependent loads a slot.
 // Where many of the slots are dead this chain is the call's time (a whole
-// warp a slot, with wider scans: 1M primitives, K = 14, 95% dead 398 us, 304
+// warp a slot, with wider scans: 1M primitives, K = 15, 95% dead 398 us, 304
 // so; 20% 174, 155), so a CTA takes 1024 slots only in scenes that give two
 // CTAs an SM that way, and down to 64 in smaller ones: 100K primitives, 20%
 // dead 46 us with 1024, 29 with 256 (5% 32, 25); 5000, 20% 33, 20 with 64.

@@ -253,8 +253,11 @@ __device__ __forceinline__ bool certain_cull_one(const PrimIn<C>& in, float belo
 // ones not culled in shared memory; then the listed ones go through the rule
 // set, one a thread, their parameters read again (in L1 and L2).
 // 300K N=7 primitives, 1.4% drawn: 31 us with every one through the rule set,
-// 17.6 us so; 200K N=6, 7% drawn: 22 -> 14.6.  Held to 64 registers, so that
-// these grids are one wave (at 80 registers 23 and 14.3 us, at 128 23 and 21).
+// 17.6 us so; 200K N=6, 7% drawn: 22 -> 14.6.  Held to 64 registers, four CTAs
+// an SM, with spills: against three at 80 the forward of one view is 1-3%
+// slower at 200K primitives, 3-10% faster at 300K, which are one wave of CTAs
+// only so, and from 600K to 2M 0-5% faster for N = 4 and 6 and equal for N = 7,
+// whether the query culls most or few.
 constexpr int kOneThreads = 256, kOnePrims = 512;
 // Below kOneMin primitives preprocess_kernel takes the scene, in CTAs of
 // kFewThreads: its grid then fills the GPU where that of kOnePrims a CTA does

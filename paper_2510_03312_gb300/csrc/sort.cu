@@ -671,8 +671,8 @@ __global__ void __launch_bounds__(kTsW * 32, 8) tile_sort_kernel(const uint2* __
 // ---------------------------------------------------------------- merge
 
 constexpr int kMgT = 512;  // threads of a merge CTA
-// chunks of long lists up to which split-list problems join segments by rank
-// (about one wave of merge CTAs, of kMergeSeg entries each)
+// chunks (of all lists over kSortChunk) up to which split-list problems join
+// segments by rank (about one wave of merge CTAs, of kMergeSeg entries each)
 constexpr uint32_t kJoinChunks = 2048;
 
 // Merges the sorted runs A = src[a0, a0 + na) and B = src[b0, b0 + nb)
